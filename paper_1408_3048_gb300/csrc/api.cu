@@ -165,7 +165,7 @@ struct PlanHolder : Plan {
     unsigned bar_absent = 0;
     unsigned long long bar_wait_ns = BARRIER_WAIT_NS;
     std::vector<mm_psd> h_psd;
-    double* grad_H = nullptr;   // [3][npsd][N+1] derivative spectra (FP64 block)
+    double* grad_H = nullptr;   // [3][npsd][split_size(N)] derivative spectra (FP64 block)
     double* grad_u = nullptr;   // [nt] P mu
     double* grad_part = nullptr;  // [K]
     int* h_flags = nullptr;     // pinned
@@ -397,11 +397,8 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
         h2d(tz.ptw, ptT.data(), ptT.size() * sizeof(T), P.stream);
         sync(P.stream);
     }
-    std::vector<T> H((size_t)P.npsd * (N + 1));
-    for (int p = 0; p < P.npsd; ++p) {
-        const std::vector<double> h = overlap_save_spectrum(P.rows[(size_t)p], N);
-        for (int64_t k = 0; k <= N; ++k) H[(size_t)p * (N + 1) + k] = (T)h[(size_t)k];
-    }
+    const std::vector<double> Hd = fold_split_spectra(P.rows, N);
+    const std::vector<T> H(Hd.begin(), Hd.end());
     tz.H = dalloc<T>(H.size());
     h2d(tz.H, H.data(), H.size() * sizeof(T), P.stream);
     sync(P.stream);   // host vectors go out of scope
@@ -435,11 +432,9 @@ static void build_toeplitz_df(Plan& P) {
         for (size_t i = 0; i < pt.size(); ++i) ptd[i] = dfl(pt[i]);
         tz.ptw = dalloc<dfl>(ptd.size());
         h2d(tz.ptw, ptd.data(), ptd.size() * sizeof(dfl), P.stream);
-        std::vector<dfl> H((size_t)P.npsd * (N + 1));
-        for (int p = 0; p < P.npsd; ++p) {
-            const std::vector<double> h = overlap_save_spectrum(P.rows[(size_t)p], N);
-            for (int64_t k = 0; k <= N; ++k) H[(size_t)p * (N + 1) + k] = dfl(h[(size_t)k]);
-        }
+        const std::vector<double> Hd = fold_split_spectra(P.rows, N);
+        std::vector<dfl> H(Hd.size());
+        for (size_t i = 0; i < Hd.size(); ++i) H[i] = dfl(Hd[i]);
         tz.H = dalloc<dfl>(H.size());
         h2d(tz.H, H.data(), H.size() * sizeof(dfl), P.stream);
         sync(P.stream);   // host vectors go out of scope
@@ -1532,16 +1527,14 @@ static void ensure_grad(PlanHolder& P) {
     if (P.grad_H != nullptr) return;
     if (P.tz64.logn == 0) throw Error{MM_ERR_ARG, "the PSD gradient needs an FP64 Toeplitz block for this lambda"};
     const int64_t N = int64_t(1) << P.tz64.logn;
-    std::vector<double> H((size_t)3 * P.npsd * (N + 1));
+    std::vector<std::vector<double>> rows((size_t)3 * P.npsd);
     for (int p = 0; p < P.npsd; ++p) {
         if (!(P.h_psd[(size_t)p].fknee > 0.0)) throw Error{MM_ERR_ARG, "the PSD gradient needs fknee > 0"};
         const auto D = toeplitz_row_derivatives(P.h_psd[(size_t)p].sigma, P.h_psd[(size_t)p].fknee,
                                                 P.h_psd[(size_t)p].alpha, P.L_grid, P.fsamp, P.lambda, P.window);
-        for (int c = 0; c < 3; ++c) {
-            const std::vector<double> h = overlap_save_spectrum(D[(size_t)c], N);
-            std::copy(h.begin(), h.end(), H.begin() + ((size_t)c * P.npsd + p) * (N + 1));
-        }
+        for (int c = 0; c < 3; ++c) rows[(size_t)c * P.npsd + p] = D[(size_t)c];
     }
+    const std::vector<double> H = fold_split_spectra(rows, N);
     P.grad_H = dalloc<double>(H.size());
     h2d(P.grad_H, H.data(), H.size() * 8, P.stream);
     P.grad_u = dalloc<double>((size_t)P.nt);
@@ -1596,7 +1589,7 @@ static void grad(PlanHolder& P, const double* d, const double* m, const double* 
         std::vector<double> part((size_t)P.K);
         for (int c = 0; c < 3; ++c) {
             ToeplitzDev tzc = P.tz64;
-            tzc.H = P.grad_H + (size_t)c * P.npsd * (N + 1);
+            tzc.H = P.grad_H + (int64_t)c * P.npsd * split_size(N);
             launch_toeplitz<double>(P, tzc, P.dbuf, nullptr, P.tod64, nullptr, s);
             launch_interval_dot(P.grad_u, P.tod64, P.ioff, P.K, P.grad_part, s);
             d2h(part.data(), P.grad_part, (size_t)P.K * 8, s);

@@ -50,7 +50,7 @@ struct ToeplitzDev {
     Tile* tiles = nullptr;   // [ntiles]
     void* twiddle = nullptr; // T[B/4 + 1]: cos(2 pi k / B)
     void* ptw = nullptr;     // T2[...]: per-pass twiddles of the N-point FFT
-    void* H = nullptr;       // T[npsd][N + 1]: kernel spectrum / N (real, even kernel)
+    void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N, folded (fold_split_spectra)
 };
 
 struct CoarseDev {
@@ -223,6 +223,9 @@ bool symbol_positive(const std::vector<double>& t);
 std::vector<std::vector<double>> toeplitz_row_derivatives(double sigma, double fknee, double alpha, int64_t L,
                                                           double fsamp, int lam, int window);
 std::vector<double> overlap_save_spectrum(const std::vector<double>& t, int64_t N);
+// values of a folded spectrum: alpha [N], beta [N/2 + 1], one of padding
+__host__ __device__ constexpr int64_t split_size(int64_t N) { return N + N / 2 + 2; }
+std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& rows, int64_t N);
 // per-pass Stockham twiddles of an N = 2^logn point FFT as interleaved (cos, sin)
 std::vector<double> pass_twiddle_table(int logn);
 double rcond_sym3(const double B[6]);

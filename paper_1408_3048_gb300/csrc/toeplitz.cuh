@@ -5,9 +5,8 @@
 // three segments of consecutive stationary intervals of one PSD (zeros between and
 // around them, at least lambda between two intervals: see Tile),
 // packs them as N complex values u_m = y_2m + i y_2m+1, runs an N-point complex FFT,
-// turns that into the spectrum of the real block (real-FFT post-processing), multiplies
-// by the real spectrum H of the even kernel (t_|k| for |k| <= lambda, laid out
-// circularly over B), converts back to the packed N-point form and inverts with the
+// multiplies by the real spectrum H of the even kernel (t_|k| for |k| <= lambda, laid out
+// circularly over B) in packed form (split_product) and inverts with the
 // same forward FFT (conjugation trick).  Outputs [lambda, lambda + nout) of the block
 // equal the truncated band product exactly (no wrap-around reaches them when
 // nout <= B - 2 lambda).
@@ -17,9 +16,9 @@
 // memory with one padding slot after every 16 complex values so that the strided stores
 // of a pass are free of bank conflicts, butterflies of a pass held in registers (in
 // place, with barriers).  Twiddles: FP32 computes them in registers (sincospif and a few
-// products); FP64 and double-float read the per-pass tables and a quarter-wave cosine
-// table cos(2 pi k / B), k = 0..B/4 (host-computed in FP64), the latter staged in
-// shared memory.
+// products); FP64 and double-float read the per-pass tables; the cross-CTA steps of the
+// cluster blocks read a quarter-wave cosine table cos(2 pi k / B), k = 0..B/4
+// (host-computed in FP64).
 //
 // The tile load can evaluate y = P x on the fly from the map (fused de-pointing); the
 // FP32 I/Q/U form reads the map packed per pixel (one 16-byte load per sample).
@@ -68,9 +67,9 @@ __device__ __forceinline__ dfl2 ldc(const dfl2* p) {
 template <typename T>
 struct TzArgs {
     const Tile* tiles;
-    const T* twiddle;      // [N/2 + 1]: cos(2 pi k / B), real-FFT split
+    const T* twiddle;      // [N/2 + 1]: cos(2 pi k / B), cross-CTA step of the cluster blocks
     const typename Cx<T>::type* ptw;  // per-pass FFT twiddles (ptw_offset)
-    const T* H;            // [npsd][N + 1]
+    const T* H;            // [npsd][split_size(N)] folded spectra
     const In<T>* y;        // time-domain input (mode 0)
     const double* yd;      // FP64 time-domain input (modes 2, 4, 5)
     const In<T>* x;        // map (gather modes)
@@ -618,44 +617,22 @@ __device__ __forceinline__ void store_out(const Tile& tile, In<T>* z, int lambda
     if (in) z[p + seg_d(tile, g)] = to_in<T>(v);
 }
 
-// Real-FFT split of the packed spectrum at the bin pair (k, N - k), product with the real
-// kernel spectrum (h1 = H[k], h2 = H[N - k]) and the merge back to packed form, returned
-// conjugated for the inverse-by-forward transform.  (cw, sw) = (cos, sin) of 2 pi k / B.
+// Spectrum product of the packed real block at the bin pair (k, N - k).  Written out, the
+// chain real-FFT split -> product with the real kernel spectrum -> merge back to packed form
+// is linear in u1 = U_k and conj(u2), u2 = U_{N-k}, with real coefficients that depend on the
+// kernel and k alone (fold_split_spectra):
+//   V_k = alpha_k u1 + i beta_k conj(u2),   V_{N-k} = alpha_{N-k} u2 + i beta_k conj(u1),
+// eight operations for the pair and no twiddle, where the chain done step by step took 44
+// and a sine and cosine per pair (one A x in FP64 on 2^22 samples at lambda = 4096: 1.003 ->
+// 0.924 ms, FP64-pipe bound; FP32 on 2^24: 219 -> 213 us).  Returned conjugated: the forward FFT of conj(V) is conj of
+// N * IFFT(V).
 template <typename T>
-__device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename Cx<T>::type u2, T cw, T sw, T h1,
-                                              T h2, typename Cx<T>::type& V1, typename Cx<T>::type& V2) {
-    using C2 = typename Cx<T>::type;
-    // E = (u1 + conj u2)/2, O = -i (u1 - conj u2)/2
-    C2 E, O;
-    E.x = (T)0.5 * (u1.x + u2.x); E.y = (T)0.5 * (u1.y - u2.y);
-    O.x = (T)0.5 * (u1.y + u2.y); O.y = (T)-0.5 * (u1.x - u2.x);
-    const C2 WO = cmul<T>(O, cw, sw);
-    C2 X1, X2;                         // X_k = E + W O, X_{N-k} = conj(E - W O)
-    X1.x = E.x + WO.x; X1.y = E.y + WO.y;
-    X2.x = E.x - WO.x; X2.y = -(E.y - WO.y);
-    C2 Z1, Z2;
-    Z1.x = h1 * X1.x; Z1.y = h1 * X1.y;
-    Z2.x = h2 * X2.x; Z2.y = h2 * X2.y;
-    // V1 = (Z1 + conj Z2)/2 + i conj(W) (Z1 - conj Z2)/2
-    // V2 = (Z2 + conj Z1)/2 - i W (Z2 - conj Z1)/2
-    C2 S1, D1, S2, D2;
-    S1.x = (T)0.5 * (Z1.x + Z2.x); S1.y = (T)0.5 * (Z1.y - Z2.y);
-    D1.x = (T)0.5 * (Z1.x - Z2.x); D1.y = (T)0.5 * (Z1.y + Z2.y);
-    S2.x = S1.x; S2.y = -S1.y;
-    D2.x = -D1.x; D2.y = D1.y;
-    {
-        const T px = cw * D1.x - sw * D1.y;   // conj(W) * D1
-        const T py = cw * D1.y + sw * D1.x;
-        V1.x = S1.x - py; V1.y = S1.y + px;   // + i (px + i py)
-    }
-    {
-        const T px = cw * D2.x + sw * D2.y;   // W * D2
-        const T py = cw * D2.y - sw * D2.x;
-        V2.x = S2.x + py; V2.y = S2.y - px;   // - i (px + i py)
-    }
-    // conjugates: the forward FFT of conj(V) is conj of N * IFFT(V)
-    V1.y = -V1.y;
-    V2.y = -V2.y;
+__device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename Cx<T>::type u2, T a1, T a2, T b,
+                                              typename Cx<T>::type& V1, typename Cx<T>::type& V2) {
+    V1.x = a1 * u1.x + b * u2.y;
+    V1.y = -(a1 * u1.y + b * u2.x);
+    V2.x = a2 * u2.x + b * u1.y;
+    V2.y = -(a2 * u2.y + b * u1.x);
 }
 
 template <typename T, int LOGN, int NT, int MODE>
@@ -663,11 +640,9 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
     griddep_wait();   // launched as a dependent launch: the previous kernel's outputs
     using C2 = typename Cx<T>::type;
     constexpr int N = 1 << LOGN;
-    constexpr int Q = N / 2;             // B/4
     if (A.done != nullptr && *(volatile const int*)A.done) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C2* a = reinterpret_cast<C2*>(smem_raw);
-    T* tab = reinterpret_cast<T*>(smem_raw + sizeof(C2) * (N + (N >> PadLog<T>::v)));
     const TileRhs tr = tile_rhs(blockIdx.x, A.R);
     const Tile tile = A.tiles[tr.tile];
     const int tid = threadIdx.x;
@@ -676,29 +651,17 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
     PfSeg next{0, 0, 0};
     if (A.pf_ahead > 0 && (int64_t)blockIdx.x + A.pf_ahead < (int64_t)gridDim.x)
         next = prefetch_seg(A, blockIdx.x + A.pf_ahead);
-    // FP32: the split twiddles are computed (sincospif), which leaves the table's 32 KB of
-    // shared memory to the L1 cache that serves the de-pointing gathers
-    if constexpr (sizeof(T) != 4)
-        for (int i = tid; i <= Q; i += NT) tab[i] = A.twiddle[i];
     load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), 0, 2 * N, tr.rhs * A.in_stride);
     __syncthreads();
     prefetch_issue<T, MODE>(A, next);
     fft_all<T, LOGN, NT, 0>(a, A.ptw);
-    // real-FFT post-processing, spectrum product, pre-processing for the inverse.
-    const T* H = A.H + (int64_t)tile.psd * (N + 1);
+    constexpr int64_t HS = split_size(N);
+    const T* al = A.H + tile.psd * HS;
+    const T* be = al + N;
     for (int k = tid; k <= N / 2; k += NT) {
         const int k2 = (N - k) & (N - 1);
-        T cw, sw;                         // W = cw - i sw = exp(-2 pi i k / B)
-        if constexpr (sizeof(T) == 4) {
-            float sv, cv;
-            sincospif((float)k * (1.f / (float)N), &sv, &cv);   // 2 pi k / B = pi k / N
-            cw = cv;
-            sw = sv;
-        } else {
-            twiddle<T, LOGN - 1>(tab, k, cw, sw);
-        }
         C2 V1, V2;
-        split_product<T>(a[pad<T>(k)], a[pad<T>(k2)], cw, sw, H[k], H[N - k], V1, V2);
+        split_product<T>(a[pad<T>(k)], a[pad<T>(k2)], al[k], al[k2], be[k], V1, V2);
         a[pad<T>(k)] = V1;
         if (k2 != k) a[pad<T>(k2)] = V2;
     }
@@ -819,7 +782,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     for (int u = 0; u < PER; ++u) a[pad<T>(u * NT + tid)] = y[u];
     __syncthreads();
     fft_all<T, LOGM, NT, 0>(a, A.ptw);
-    const T* H = A.H + (int64_t)tile.psd * (N + 1);
+    constexpr int64_t HS = split_size(N);
+    const T* al = A.H + tile.psd * HS;
+    const T* be = al + N;
     const int prank = (CL - rank) % CL;
     if (prank == rank) {
         // partner bins inside this CTA: process each pair once
@@ -827,10 +792,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
         for (int k1 = tid; k1 < npairs; k1 += NT) {
             const int k = CL * k1 + rank;
             const int p = rank == 0 ? ((M - k1) & (M - 1)) : (M - 1 - k1);
-            T cw, sw;
-            twiddle<T, LOGQ>(A.twiddle, k, cw, sw);
+            const int k2 = (N - k) & (N - 1);
             C2 V1, V2;
-            split_product<T>(a[pad<T>(k1)], a[pad<T>(p)], cw, sw, H[k], H[N - k], V1, V2);
+            split_product<T>(a[pad<T>(k1)], a[pad<T>(p)], al[k], al[k2], be[k < k2 ? k : k2], V1, V2);
             a[pad<T>(k1)] = V1;
             if (p != k1) a[pad<T>(p)] = V2;
         }
@@ -844,10 +808,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
         for (int u = 0; u < PER; ++u) {
             const int k1 = u * NT + tid;
             const int k = CL * k1 + rank;
-            T cw, sw;
-            twiddle<T, LOGQ>(A.twiddle, k, cw, sw);
             C2 V2;
-            split_product<T>(a[pad<T>(k1)], part[prank][pad<T>(M - 1 - k1)], cw, sw, H[k], H[N - k], vo[u], V2);
+            split_product<T>(a[pad<T>(k1)], part[prank][pad<T>(M - 1 - k1)], al[k], al[N - k],
+                             be[k < N - k ? k : N - k], vo[u], V2);
         }
         cl.sync();
 #pragma unroll
@@ -924,9 +887,7 @@ void launch_mode_cl(const TzArgs<T>& A, int ntiles, int mode, cudaStream_t s) {
 template <typename T>
 size_t toeplitz_smem_bytes_impl(int logn) {
     const size_t N = size_t(1) << logn;
-    // the FP32 kernel computes its split twiddles and holds no cosine table
-    const size_t table = sizeof(T) == 4 ? 0 : sizeof(T) * (N / 2 + 1);
-    return sizeof(typename Cx<T>::type) * (N + (N >> PadLog<T>::v)) + table;
+    return sizeof(typename Cx<T>::type) * (N + (N >> PadLog<T>::v));
 }
 
 template <typename T, int LOGN, int MODE>
