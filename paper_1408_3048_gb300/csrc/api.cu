@@ -35,7 +35,7 @@ void check_cuda(cudaError_t e, const char* what) {
     }
 }
 
-void ensure_smem_attr(const void* kern, int bytes, const char* what) {
+void ensure_smem_attr(const void* kern, int bytes, const char* what, int carveout) {
     static std::mutex mu;
     static std::set<std::pair<const void*, int>> done;   // (kernel, device)
     int dev = 0;
@@ -43,6 +43,7 @@ void ensure_smem_attr(const void* kern, int bytes, const char* what) {
     std::lock_guard<std::mutex> lock(mu);
     if (done.count({kern, dev})) return;
     check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes), what);
+    if (carveout >= 0) check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carveout), what);
     done.insert({kern, dev});
 }
 
@@ -195,6 +196,9 @@ static void free_tz(ToeplitzDev& t) {
     dfree(t.twiddle);
     dfree(t.ptw);
     dfree(t.H);
+    dfree(t.ws_tab);
+    dfree(t.ws_H);
+    dfree(t.ws_scratch);
     t = ToeplitzDev{};
 }
 
@@ -274,9 +278,15 @@ double block_weight<float>(int logn) {
 // one sequence, which saves the partly filled last tile of every interval but one.  A run
 // is packed only when that gives fewer tiles and no tile needs more than TILE_SEGS
 // segments; otherwise each interval is tiled on its own (one segment per tile).
+// Outputs of a full tile: B - 2 lambda, rounded down to a multiple of 4 where that leaves any
+// (the distance of two windows is then one that the FP32 kernel copies between them).
+static int64_t tile_outputs(int64_t B, int64_t lam) {
+    const int64_t v = B - 2 * lam;
+    return v >= 4 ? v & ~int64_t(3) : v;
+}
 static std::vector<Tile> make_tiles(const Plan& P, int64_t B) {
     const int64_t lam = P.lambda;
-    const int64_t Lv = B - 2 * lam;
+    const int64_t Lv = tile_outputs(B, lam);
     std::vector<Tile> out;
     auto tile_run = [&](int i0, int i1, std::vector<Tile>& dst) -> bool {
         // virtual start of each interval of the run [i0, i1)
@@ -284,6 +294,9 @@ static std::vector<Tile> make_tiles(const Plan& P, int64_t B) {
         int64_t vlen = 0;
         for (int i = i0; i < i1; ++i) {
             if (i > i0) vlen += lam;
+            // up to three more zeros, so that the shift from position to time is a multiple of
+            // four: the FP32 kernel then stores four outputs as one 16-byte word
+            vlen += (P.h_ioff[i] - lam - vlen) & 3;
             V[(size_t)(i - i0)] = vlen;
             vlen += P.h_ioff[i + 1] - P.h_ioff[i];
         }
@@ -310,6 +323,8 @@ static std::vector<Tile> make_tiles(const Plan& P, int64_t B) {
             }
             t.nout = (int32_t)std::min<int64_t>(Lv, vlen - k * Lv);
             t.psd = P.h_ipsd[i0];
+            t.cont = k > 0 && Lv % 4 == 0 ? (int32_t)Lv : 0;
+            t.unused = 0;
             dst.push_back(t);
         }
         return true;
@@ -384,11 +399,14 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
     tz.ntiles = (int)tiles.size();
     tz.tiles = dalloc<Tile>(tiles.size());
     h2d(tz.tiles, tiles.data(), tiles.size() * sizeof(Tile), P.stream);
-    std::vector<T> tw((size_t)(B / 4 + 1));
-    for (int64_t k = 0; k <= B / 4; ++k) tw[(size_t)k] = (T)std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B);
-    tz.twiddle = dalloc<T>(tw.size());
-    h2d(tz.twiddle, tw.data(), tw.size() * sizeof(T), P.stream);
-    {
+    if (tz.cluster > 1) {   // cross-CTA twiddles
+        std::vector<T> tw((size_t)(B / 4 + 1));
+        for (int64_t k = 0; k <= B / 4; ++k) tw[(size_t)k] = (T)std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B);
+        tz.twiddle = dalloc<T>(tw.size());
+        h2d(tz.twiddle, tw.data(), tw.size() * sizeof(T), P.stream);
+        sync(P.stream);
+    }
+    if constexpr (sizeof(T) == 8) {   // pass twiddles (FP32 forms its own)
         // the cluster kernel runs local FFTs of half the length
         const int lc = tz.cluster == 4 ? 2 : (tz.cluster == 2 ? 1 : 0);
         const std::vector<double> pt = pass_twiddle_table(tz.logn - lc);
@@ -398,6 +416,18 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
         sync(P.stream);
     }
     const std::vector<double> Hd = fold_split_spectra(P.rows, N);
+    if constexpr (sizeof(T) == 4) {
+        if (tz.cluster == 1 && ws_supported(tz.logn)) {
+            const std::vector<float> tab = ws_tables(tz.logn), Hw = ws_spectra(Hd, P.npsd, tz.logn);
+            tz.ws_tab = dalloc<float>(tab.size());
+            h2d(tz.ws_tab, tab.data(), tab.size() * 4, P.stream);
+            tz.ws_H = dalloc<float>(Hw.size());
+            h2d(tz.ws_H, Hw.data(), Hw.size() * 4, P.stream);
+            tz.ws_scratch = dalloc<float>(ws_scratch_floats(tz.logn, P.num_sms));
+            sync(P.stream);
+            return;
+        }
+    }
     const std::vector<T> H(Hd.begin(), Hd.end());
     tz.H = dalloc<T>(H.size());
     h2d(tz.H, H.data(), H.size() * sizeof(T), P.stream);
@@ -422,10 +452,12 @@ static void build_toeplitz_df(Plan& P) {
         tz.tiles = dalloc<Tile>((size_t)tz.ntiles);
         check_cuda(cudaMemcpyAsync(tz.tiles, src.tiles, (size_t)tz.ntiles * sizeof(Tile), cudaMemcpyDeviceToDevice,
                                    P.stream), "copy tiles");
-        std::vector<dfl> tw((size_t)(B / 4 + 1));
-        for (int64_t k = 0; k <= B / 4; ++k) tw[(size_t)k] = dfl(std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B));
-        tz.twiddle = dalloc<dfl>(tw.size());
-        h2d(tz.twiddle, tw.data(), tw.size() * sizeof(dfl), P.stream);
+        std::vector<dfl> tw(tz.cluster > 1 ? (size_t)(B / 4 + 1) : 1);
+        if (tz.cluster > 1) {   // cross-CTA twiddles
+            for (int64_t k = 0; k <= B / 4; ++k) tw[(size_t)k] = dfl(std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B));
+            tz.twiddle = dalloc<dfl>(tw.size());
+            h2d(tz.twiddle, tw.data(), tw.size() * sizeof(dfl), P.stream);
+        }
         const int lc = tz.cluster == 4 ? 2 : (tz.cluster == 2 ? 1 : 0);
         const std::vector<double> pt = pass_twiddle_table(tz.logn - lc);
         std::vector<dfl> ptd(pt.size());
@@ -625,8 +657,9 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
     }
     // --- device buffers
     cudaStream_t s = P.stream;
-    P.pixc = dalloc<int32_t>((size_t)nt);
+    P.pixc = dalloc<int32_t>((size_t)nt + PIXC_PAD);
     h2d(P.pixc, pixc.data(), (size_t)nt * 4, s);
+    check_cuda(cudaMemsetAsync(P.pixc + nt, 0xff, PIXC_PAD * 4, s), "memset");
     P.csr_off = dalloc<int32_t>(off.size());
     h2d(P.csr_off, off.data(), off.size() * 4, s);
     P.tsort = dalloc<int32_t>((size_t)P.nkept);

@@ -12,6 +12,10 @@
 
 namespace mm {
 
+// entries of -1 behind the pixel indices: a gather that asks for its next indices ahead of
+// time reads up to this many past the last sample
+constexpr int PIXC_PAD = 8192;
+
 // ---------------------------------------------------------------------------------
 // Overlap-save tile of the single-right-hand-side Toeplitz kernels: a block of B real
 // positions holding up to TILE_SEGS segments of samples.  Segment g covers block positions
@@ -29,6 +33,8 @@ struct Tile {
     int32_t pe[TILE_SEGS];
     int32_t nout;
     int32_t psd;
+    int32_t cont;   // positions from the window of the tile before, of the same run, to this one's (0: none)
+    int32_t unused;
 };
 
 // Tile of the batched kernels: block of B real samples [in0, in0 + B) of one interval
@@ -48,8 +54,13 @@ struct ToeplitzDev {
     int cluster = 1;         // CTAs per tile (2 or 4: split across a thread-block cluster)
     int ntiles = 0;
     Tile* tiles = nullptr;   // [ntiles]
-    void* twiddle = nullptr; // T[B/4 + 1]: cos(2 pi k / B)
-    void* ptw = nullptr;     // T2[...]: per-pass twiddles of the N-point FFT
+    void* twiddle = nullptr; // T[B/4 + 1]: cos(2 pi k / B) (cluster blocks)
+    void* ptw = nullptr;     // T2[...]: per-pass twiddles of the N-point FFT (not FP32)
+    // FP32 blocks of 2^14 and 2^15 reals (toeplitz_ws.cu): twiddle tables, folded spectra in
+    // the kernel's order, and two input buffers of B floats per resident CTA
+    void* ws_tab = nullptr;
+    void* ws_H = nullptr;
+    float* ws_scratch = nullptr;
     void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N, folded (fold_split_spectra)
 };
 
@@ -175,8 +186,9 @@ struct Error {
 
 void check_cuda(cudaError_t e, const char* what);   // throws Error{MM_ERR_CUDA}
 // cudaFuncSetAttribute(kern, MaxDynamicSharedMemorySize, bytes) once per kernel and
-// device (thread-safe; the attribute is per device, so a second GPU gets its own call)
-void ensure_smem_attr(const void* kern, int bytes, const char* what);
+// device (thread-safe; the attribute is per device, so a second GPU gets its own call);
+// carveout: also the preferred shared-memory share of the SM's 228 KB in percent (-1: default)
+void ensure_smem_attr(const void* kern, int bytes, const char* what, int carveout = -1);
 // Runs f and turns what it throws into a status: sets P->err (P may be null) and the
 // calling thread's last-error message (mm_last_error(NULL)).  Nothing leaves it.
 mm_status run_guarded(Plan* P, void (*f)(void*), void* ctx);
@@ -253,6 +265,10 @@ void launch_toeplitz_df(const Plan& P, const double* y, const double* d, const d
 // P.map4 (one small kernel), else P.map4 already holds x (the FP32 PCG kernels keep it)
 void launch_toeplitz_f32_packed(const Plan& P, const float* x, bool pack, float* z, const int* done,
                                 cudaStream_t s);
+bool ws_supported(int logn);
+std::vector<float> ws_tables(int logn);
+std::vector<float> ws_spectra(const std::vector<double>& folded, int npsd, int logn);
+size_t ws_scratch_floats(int logn, int num_sms);
 template <typename T>
 size_t toeplitz_smem_bytes(int logn);
 template <typename T>

@@ -578,9 +578,8 @@ struct PfSeg {
 };
 
 template <typename T>
-__device__ __forceinline__ PfSeg prefetch_seg(const TzArgs<T>& A, int cid) {
+__device__ __forceinline__ PfSeg prefetch_seg(const TzArgs<T>& A, int cid, int g) {
     PfSeg sg{0, 0, 0};
-    const int g = threadIdx.x;
     if (g >= TILE_SEGS) return sg;
     const TileRhs tr = tile_rhs(cid, A.R);
     const Tile& tl = A.tiles[tr.tile];
@@ -650,7 +649,7 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
     // are not: a prefetch racing the CTA's own loads measured slower than none)
     PfSeg next{0, 0, 0};
     if (A.pf_ahead > 0 && (int64_t)blockIdx.x + A.pf_ahead < (int64_t)gridDim.x)
-        next = prefetch_seg(A, blockIdx.x + A.pf_ahead);
+        next = prefetch_seg(A, blockIdx.x + A.pf_ahead, threadIdx.x);
     load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), 0, 2 * N, tr.rhs * A.in_stride);
     __syncthreads();
     prefetch_issue<T, MODE>(A, next);

@@ -9,8 +9,10 @@ size_t toeplitz_smem_bytes<float>(int logn) { return toeplitz_smem_bytes_impl<fl
 template <>
 int toeplitz_max_logn<float>() { return 14; }
 
+void launch_toeplitz_ws(const TzArgs<float>& A, const ToeplitzDev& tz, int num_sms, int mode, cudaStream_t s);
+
 // Launch of the instance for the plan's FP32 block (single CTA or 2- / 4-CTA cluster).
-static void dispatch_f32(const TzArgs<float>& A, const ToeplitzDev& tz, int mode, cudaStream_t s) {
+static void dispatch_f32(const TzArgs<float>& A, const ToeplitzDev& tz, int num_sms, int mode, cudaStream_t s) {
     if (tz.cluster == 2 && tz.logn == 15) {
         launch_mode_cl<float, 14, 2>(A, tz.ntiles, mode, s);
         return;
@@ -26,8 +28,8 @@ static void dispatch_f32(const TzArgs<float>& A, const ToeplitzDev& tz, int mode
         case 10: launch_mode<float, 10>(A, tz.ntiles, mode, s); break;
         case 11: launch_mode<float, 11>(A, tz.ntiles, mode, s); break;
         case 12: launch_mode<float, 12>(A, tz.ntiles, mode, s); break;
-        case 13: launch_mode<float, 13>(A, tz.ntiles, mode, s); break;
-        case 14: launch_mode<float, 14>(A, tz.ntiles, mode, s); break;
+        case 13:
+        case 14: launch_toeplitz_ws(A, tz, num_sms, mode, s); break;
         default: throw Error{MM_ERR_ARG, "unsupported FFT length"};
     }
 }
@@ -57,7 +59,7 @@ void launch_toeplitz_any<float>(const Plan& P, const ToeplitzDev& tz, const floa
     A.out_stride = out_stride;
     A.pf_ahead = P.num_sms;
     const int mode = y != nullptr ? 0 : (yd != nullptr ? (x == nullptr ? 2 : (P.ncomp == 1 ? 4 : 5)) : (P.ncomp == 1 ? 1 : 3));
-    dispatch_f32(A, tz, mode, s);
+    dispatch_f32(A, tz, P.num_sms, mode, s);
 }
 
 template <>
@@ -109,7 +111,7 @@ void launch_toeplitz_f32_packed(const Plan& P, const float* x, bool pack, float*
     A.out_stride = 0;
     A.pf_ahead = P.num_sms;
     A.x4 = P.map4;
-    dispatch_f32(A, tz, 3, s);
+    dispatch_f32(A, tz, P.num_sms, 3, s);
 }
 
 }  // namespace mm
