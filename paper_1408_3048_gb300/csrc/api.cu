@@ -214,7 +214,8 @@ static void free_coarse(CoarseDev& c) {
 static void destroy_plan(PlanHolder* P) {
     if (P == nullptr) return;
     for (void* p : {(void*)P->pixc, (void*)P->w64, (void*)P->w32, (void*)P->csr_off, (void*)P->tsort,
-                    (void*)P->wsort64, (void*)P->wsort32, (void*)P->asort32, (void*)P->ioff, (void*)P->ipsd, (void*)P->t0,
+                    (void*)P->wsort64, (void*)P->wsort32, (void*)P->asort32, (void*)P->sl_off, (void*)P->sl_t,
+                    (void*)P->sl_w64, (void*)P->sl_w32, (void*)P->sl_ang, (void*)P->ioff, (void*)P->ipsd, (void*)P->t0,
                     (void*)P->bd64, (void*)P->bd32, (void*)P->tod64, (void*)P->tod32, (void*)P->map4, (void*)P->dbuf,
                     (void*)P->b64, (void*)P->d_dot, (void*)P->x64, (void*)P->r64, (void*)P->ax64,
                     (void*)P->grad_H, (void*)P->grad_u, (void*)P->grad_part})
@@ -525,6 +526,71 @@ static void autotune_toeplitz(PlanHolder& P, ToeplitzDev& tz, T* tod, const T* z
     }
 }
 
+static void free_sliced(Plan& P) {
+    for (void* p : {(void*)P.sl_off, (void*)P.sl_t, (void*)P.sl_w64, (void*)P.sl_w32, (void*)P.sl_ang}) dfree(p);
+    P.sl_off = P.sl_t = nullptr;
+    P.sl_w64 = nullptr;
+    P.sl_w32 = nullptr;
+    P.sl_ang = nullptr;
+}
+
+// Frees the sorted weights that the 32-lane scatters no longer read.
+static void free_sorted_weights(Plan& P) {
+    if (P.sl_off == nullptr) return;
+    dfree(P.wsort64);
+    P.wsort64 = nullptr;
+    if (!P.sl_f32) return;
+    dfree(P.wsort32);
+    dfree(P.asort32);
+    P.wsort32 = nullptr;
+    P.asort32 = nullptr;
+}
+
+// The sliced layout of the scatter, unless its padding (a slice is as long as its longest
+// pixel, in fours) costs more than half as many entries again: its time is its bytes, the
+// 32-lane form's is about twice that (scatter.cu), so up to there it is ahead.  The FP32
+// I/Q/U scatter of one right-hand side keeps the 32-lane form where that has four or more
+// loads a lane in flight for every pixel (128 samples), pixels enough to fill the chip and a
+// time-domain array that fits the L2 cache: 47.6 us against 52.8 on 65536 pixels of 256.
+static void build_sliced(Plan& P) {
+    constexpr int PIX = 8;
+    if (P.npix_obs == 0) return;
+    const int32_t ns = (P.npix_obs + PIX - 1) / PIX;
+    std::vector<int32_t> off((size_t)ns + 1, 0);
+    int64_t steps = 0, used = 0;   // used: entries of the pixels there are (the last slice may miss some)
+    for (int32_t s = 0; s < ns; ++s) {
+        const int32_t q0 = s * PIX, q1 = std::min(P.npix_obs, q0 + PIX);
+        int32_t most = 0;
+        for (int32_t q = q0; q < q1; ++q) most = std::max(most, P.h_hits[(size_t)q]);
+        steps += (most + 3) / 4;
+        used += (int64_t)((most + 3) / 4) * 4 * (q1 - q0);
+        if (used > P.nkept + P.nkept / 2 + 4096 || steps * 32 > 4 * P.nkept + 4096) return;
+        off[(size_t)s + 1] = (int32_t)steps;
+    }
+    P.sl_count = ns;
+    P.sl_steps = steps;
+    P.sl_f32 = P.ncomp == 1 || P.nkept < (int64_t)128 * P.npix_obs || P.npix_obs < P.num_sms * 64 || P.nt > (1 << 25);
+    const size_t e = (size_t)steps * 32 + SL_PAD;
+    try {
+        P.sl_off = dalloc<int32_t>(off.size());
+        h2d(P.sl_off, off.data(), off.size() * 4, P.stream);
+        P.sl_t = dalloc<int32_t>(e);
+        if (P.ncomp == 3) {
+            P.sl_w64 = dalloc<double2>(e);
+            P.sl_w32 = dalloc<float2>(e);
+            if (P.asort32 != nullptr && P.sl_f32) P.sl_ang = dalloc<float>(e);
+        }
+        for (auto [p, b] : {std::pair<void*, size_t>{P.sl_t, 4}, {P.sl_w64, 16}, {P.sl_w32, 8}, {P.sl_ang, 4}})
+            if (p != nullptr)
+                check_cuda(cudaMemsetAsync(static_cast<char*>(p) + (e - SL_PAD) * b, 0, SL_PAD * b, P.stream), "memset");
+        launch_slice_fill(P, P.sl_t, P.sl_w64, P.sl_w32, P.sl_ang, P.stream);
+        sync(P.stream);   // the host array goes out of scope
+    } catch (...) {
+        free_sliced(P);
+        throw;
+    }
+}
+
 static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t npix_sky, const double* weights,
                        const int64_t* ioff, int32_t K, const int32_t* ipsd, const mm_psd* psd, int32_t npsd,
                        const mm_opts* o) {
@@ -730,7 +796,7 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
     g.n = P.n;
     g.nblocks = std::max(1, std::min(pcg_max_blocks(P.num_sms), (P.npix_obs + 31) / 32));
     g.partial = dalloc<double>((size_t)g.nblocks * PSTRIDE);
-    g.sc_part = dalloc<double>((size_t)scatter_blocks(P));   // 32 lanes per pixel: the most blocks
+    g.sc_part = dalloc<double>((size_t)P.num_sms * SL_BLOCKS);   // the most blocks of any scatter
     g.sc_count = dalloc<unsigned>(1);
     check_cuda(cudaMemsetAsync(g.sc_count, 0, 4, s), "memset");
     g.scal = dalloc<double>(16);
@@ -750,6 +816,8 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
             throw Error{MM_ERR_ARG, "scatter_lanes must be 0, 32, 16 or 8"};
         P.scatter_lpp = o->scatter_lanes;
     }
+    // the sliced scatter, unless a lane count was asked for
+    if (o->scatter_lanes == 0 && !P.autotune) build_sliced(P);
     if (P.autotune) {
         // zero maps for the timed launches (x64 / the first half of r64 as FP32)
         check_cuda(cudaMemsetAsync(P.x64, 0, (size_t)P.n * 8, s), "memset");
@@ -769,8 +837,14 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
                 if (P.tuned_scatter_ms[i] < P.tuned_scatter_ms[best]) best = i;
             }
             P.scatter_lpp = lpp[best];
+            build_sliced(P);
+            if (P.sl_off != nullptr && P.sl_f32)
+                P.sl_f32 = time_launches(
+                               P, [&] { launch_scatter<float>(P, P.tod32, reinterpret_cast<float*>(P.r64), nullptr, s); },
+                               5) <= P.tuned_scatter_ms[best];
         }
     }
+    free_sorted_weights(P);
     build_toeplitz_df(P);
     sync(s);
 }

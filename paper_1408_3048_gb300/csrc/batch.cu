@@ -296,6 +296,7 @@ __global__ void batch_scatter_kernel(const int32_t* __restrict__ off, const int3
 
 void launch_batch_scatter(const Plan& P, const float* Z, float* W, int R, const int* done, cudaStream_t s) {
     if (P.npix_obs == 0) return;
+    if (P.sl_off != nullptr) return launch_batch_scatter_sliced(P, Z, W, R, done, s);
     const int th = 256;
     int g = (P.npix_obs + 7) / 8;
     if (g > P.num_sms * 32) g = P.num_sms * 32;

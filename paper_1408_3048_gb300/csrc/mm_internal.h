@@ -15,6 +15,9 @@ namespace mm {
 // entries of -1 behind the pixel indices: a gather that asks for its next indices ahead of
 // time reads up to this many past the last sample
 constexpr int PIXC_PAD = 8192;
+// entries behind the sliced scatter's last step that its last batches read and leave out
+constexpr int SL_PAD = 1024;
+constexpr int SL_BLOCKS = 32;   // blocks of a scatter per SM, at most
 
 // ---------------------------------------------------------------------------------
 // Overlap-save tile of the single-right-hand-side Toeplitz kernels: a block of B real
@@ -146,6 +149,17 @@ struct Plan {
     float2* wsort32 = nullptr;     // [nkept]
     float* asort32 = nullptr;      // [nkept] angle / pi of the sorted weights when every weight
                                    // pair has unit norm (the FP32 scatter reads 4 bytes, not 8)
+    // sliced layout of the sorted samples (scatter.cu), or null: slices of eight pixels, step j
+    // of a slice = 32 entries (four samples of each of its pixels); the sorted weight arrays
+    // above that no scatter reads any more are then freed once the plan is built
+    bool sl_f32 = false;           // the FP32 scatter of one right-hand side uses it too
+    int32_t sl_count = 0;          // slices
+    int64_t sl_steps = 0;          // steps in all
+    int32_t* sl_off = nullptr;     // [sl_count + 1] first step
+    int32_t* sl_t = nullptr;       // [sl_steps][32] sample index, -1: none
+    double2* sl_w64 = nullptr;     // [sl_steps][32] weights (pol)
+    float2* sl_w32 = nullptr;
+    float* sl_ang = nullptr;       // angles, where asort32 exists
     int64_t* ioff = nullptr;       // [K+1]
     int32_t* ipsd = nullptr;       // [K]
     double* t0 = nullptr;          // [npsd] diagonal of each row
@@ -281,11 +295,18 @@ template <typename T>
 void launch_scatter(const Plan& P, const T* z, T* w, const int* done, cudaStream_t s);
 // w = P^T z and, fused, *pq = p^T w (FP64, fixed summation order: warp partials over their
 // pixels, block partials in part[], summed in block order by the last block to finish,
-// which also resets *count to 0).  part holds scatter_blocks(P) doubles.
+// which also resets *count to 0).  part holds SL_BLOCKS doubles per SM.
 template <typename T>
 void launch_scatter_dot(const Plan& P, const T* z, T* w, const T* p, double* part, unsigned* count, double* pq,
                         const int* done, cudaStream_t s);
 int scatter_blocks(const Plan& P);
+// the same from the sliced layout (P.sl_off != nullptr); p null: no dot product
+void launch_slice_fill(const Plan& P, int32_t* st, double2* sw64, float2* sw32, float* sang, cudaStream_t s);
+template <typename T>
+void launch_scatter_sliced(const Plan& P, const T* z, T* w, const T* p, double* part, unsigned* count, double* pq,
+                           const int* done, cudaStream_t s);
+void launch_batch_scatter_sliced(const Plan& P, const float* Z, float* W, int R, const int* done, cudaStream_t s);
+int sliced_blocks(const Plan& P, int wpb, int S);
 void launch_bd_build(const Plan& P, double* bd64, float* bd32, cudaStream_t s);
 // merged a priori coarse space Z_S (Sec. 3.3.1), r groups of consecutive intervals, into
 // Z [r][n] FP64 (zeroed here)

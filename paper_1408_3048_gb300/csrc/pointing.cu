@@ -289,8 +289,12 @@ static void scatter_launch(const Plan& P, const T* z, T* w, const int* done, Sca
 }
 
 template <typename T>
+static bool use_sliced(const Plan& P) { return P.sl_off != nullptr && (sizeof(T) == 8 || P.sl_f32); }
+
+template <typename T>
 void launch_scatter(const Plan& P, const T* z, T* w, const int* done, cudaStream_t s) {
     if (P.npix_obs == 0) return;
+    if (use_sliced<T>(P)) return launch_scatter_sliced<T>(P, z, w, nullptr, nullptr, nullptr, nullptr, done, s);
     scatter_launch<T, false>(P, z, w, done, ScatterDot{nullptr, nullptr, nullptr, nullptr}, s);
 }
 template void launch_scatter<double>(const Plan&, const double*, double*, const int*, cudaStream_t);
@@ -300,6 +304,7 @@ template <typename T>
 void launch_scatter_dot(const Plan& P, const T* z, T* w, const T* p, double* part, unsigned* count, double* pq,
                         const int* done, cudaStream_t s) {
     if (P.npix_obs == 0) throw Error{MM_ERR_ARG, "no observed pixels"};
+    if (use_sliced<T>(P)) return launch_scatter_sliced<T>(P, z, w, p, part, count, pq, done, s);
     scatter_launch<T, true>(P, z, w, done, ScatterDot{p, part, count, pq}, s);
 }
 template void launch_scatter_dot<double>(const Plan&, const double*, double*, const double*, double*, unsigned*,
