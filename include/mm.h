@@ -154,8 +154,8 @@ mm_status mm_scatter_config(mm_plan_t plan, int32_t* lanes_per_pixel, float* ms)
  *   kind  (host, in/out) in: -1 = choose, 0, 1 or 2 = use that form; out: the form in use.
  *         0: two right-hand sides per complex FFT of 2^log2_block points (real kernel
  *         spectrum: real and imaginary parts convolve independently);
- *         1: one real FFT per right-hand side with the FP32 block of mm_plan_info, the
- *         right-hand side as the fastest grid index;
+ *         1: one real FFT per right-hand side, with the FP32 block of mm_plan_info or (where
+ *         neither that block nor autotuning was asked for) one better for R of them;
  *         2: the band product as a dense contraction on the tensor cores (tcgen05 MMAs in
  *         FP16 on operands split as hi + 2^-11 lo after power-of-two scaling, FP32
  *         accumulators in tensor memory; 128-row tiles, window 128 + 2 lambda; the maps

@@ -129,6 +129,7 @@ enum { BATCH_PAIR = 0, BATCH_REAL = 1, BATCH_TENSOR = 2 };
 struct BatchState {
     int kind = -1;                // BATCH_PAIR / BATCH_REAL / BATCH_TENSOR, -1 before the first call
     float tuned_ms[3] = {};       // timed forms (autotuning), 0 when not timed
+    ToeplitzDev tz;               // real form: its own FP32 block, where the plan's is not the best for R
     int logb = 0;                 // complex FFT length of the pair kernel
     int ntiles = 0;
     SpanTile* tiles = nullptr;
@@ -176,6 +177,7 @@ struct PlanHolder : Plan {
     double* r64 = nullptr;      // [n] refinement residual
     double* ax64 = nullptr;     // [n]
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
+    bool forced_f32 = false;    // the caller fixed the FP32 block
     bool autotune = false;      // measured block / batched-kernel choice (mm_opts.autotune)
     float tuned_ms64[16] = {};  // timed candidates by logn - 8 (0: not tried)
     float tuned_ms32[16] = {};
@@ -240,6 +242,7 @@ static void destroy_plan(PlanHolder* P) {
     }
     for (auto e : P->prof.pool) (void)cudaEventDestroy(e);
     BatchState& bt = P->batch;
+    free_tz(bt.tz);
     if (bt.graph) (void)cudaGraphExecDestroy(bt.graph);
     for (void* p : {(void*)bt.tiles, (void*)bt.H, (void*)bt.ptw, (void*)bt.twiddle, (void*)bt.x, (void*)bt.r,
                     (void*)bt.p, (void*)bt.q, (void*)bt.z,
@@ -251,25 +254,38 @@ static void destroy_plan(PlanHolder* P) {
     delete P;
 }
 
-// Cost of a block relative to its FFT operation count, from launch timings of every
-// admissible block on polarised scans of 2^24-2^25 samples with lambda = 1024, 4096,
-// 8192 and 16384.  FP64 kernels are bound by the FP64 pipe, so the cross-CTA steps of a
-// 2-CTA cluster cost little; the largest single-CTA FP64 block (2^14 reals) runs one
-// 512-thread CTA per SM.  FP32 kernels are bound by shared-memory and L1 latency, where
-// the cluster steps (distributed shared memory) cost more.  The batched complex-pair
-// blocks are FP32 and take the FP32 weights by cluster size.
-static double fp32_cluster_weight(int cluster) { return cluster == 4 ? 3.3 : (cluster == 2 ? 1.6 : 1.0); }
+// Time of a launch over `tiles` overlap-save tiles of a block, in microseconds, from timings of
+// every block on scans of 2^14 to 2^26 samples with lambda = 32 to 16384 (the blocks it picks
+// were within 5 % of the fastest in 43 of 46 of them).
+//
+// FP64 and double-float: a tile keeps an SM's pipe busy for `per`, alone it takes `lat`
+// (latency of its chain of passes where that is longer); tiles go round the SMs, the cluster
+// blocks' round groups of 2 and 4.  FP32 up to 2^13 reals: several CTAs per SM, a start and a
+// slope per tile and SM.  2^14 and 2^15 reals (toeplitz_ws.cu): persistent CTAs, two or one
+// per SM, a first gather and then rounds.
+struct BlockTime {
+    double lat, per;
+};
+static constexpr BlockTime TIME_F64[] = {{27, 4.6}, {49, 11.2}, {54, 22.4}, {61, 47}, {108, 112}, {222, 228}, {263, 263}, {340, 345}};
+static constexpr BlockTime TIME_DF[] = {{23, 2.0}, {49, 6.0}, {51, 13.1}, {54, 23}, {66, 65}, {83, 141}, {118, 152}, {210, 228}};
+static constexpr BlockTime TIME_F32_T[] = {{3.5, 0.32}, {8, 0.57}, {8, 1.1}, {8, 2.2}, {8, 4.4}, {14, 17}, {6, 21}, {41, 43.7}, {71, 72}};
+static constexpr BlockTime TIME_F32_IQU[] = {{5, 0.5}, {11, 0.6}, {11, 1.2}, {11, 2.35}, {12, 4.9}, {14, 20}, {6, 23.5}, {41, 43.7}, {71, 72}};
+
 template <typename T>
-static double block_weight(int logn);
-template <>
-double block_weight<double>(int logn) { return logn >= 15 ? 2.0 : (logn == 14 ? 1.2 : (logn == 13 ? 1.12 : 1.0)); }
-// FP32 single-CTA blocks below 2^15 reals run several CTAs per SM (1024 threads in all),
-// which hides part of their gathers: measured on the 2^24-sample I/Q/U scan at lambda =
-// 512 .. 8192, their time per unit of the model falls with the block.
-template <>
-double block_weight<float>(int logn) {
-    if (logn >= 15) return fp32_cluster_weight(logn >= 16 ? 4 : 2);
-    return logn == 14 ? 1.0 : (logn == 13 ? 0.87 : (logn == 12 ? 0.83 : (logn == 11 ? 0.72 : 0.67)));
+static double block_us(const Plan& P, int logn, int64_t tiles) {
+    constexpr bool F32 = sizeof(T) == 4;
+    const BlockTime* tab = F32 ? (P.ncomp == 1 ? TIME_F32_T : TIME_F32_IQU)
+                               : (std::is_same<T, double>::value ? TIME_F64 : TIME_DF);
+    const BlockTime b = tab[logn - 8];
+    const int over = logn - toeplitz_max_logn<T>();
+    // four-CTA clusters do not fill the chip (8 of 152 SMs are left over, measured)
+    const int64_t slots = over <= 0 ? P.num_sms : over == 1 ? P.num_sms / 2 : (P.num_sms - 8) / 4;
+    if (F32 && over <= 0) {
+        if (logn <= 12) return b.lat + b.per * std::max(1.0, (double)tiles / (double)slots);
+        const int64_t ctas = slots << (14 - logn);
+        return b.lat + b.per * (logn == 13 && tiles <= slots ? 0.25 : (double)((tiles + ctas - 1) / ctas));
+    }
+    return std::max(b.lat, (double)((tiles + slots - 1) / slots) * b.per);
 }
 
 // Overlap-save tiles of blocks of B real positions (B - 2 lambda valid outputs each) for
@@ -344,8 +360,11 @@ static std::vector<Tile> make_tiles(const Plan& P, int64_t B) {
     return out;
 }
 
-static int64_t overlap_tiles(const Plan& P, int64_t Lv) {
-    return (int64_t)make_tiles(P, Lv + 2 * (int64_t)P.lambda).size();
+// Number of tiles of a block, kept per plan while it is built (three arithmetics ask).
+static int64_t overlap_tiles(const Plan& P, int logn) {
+    int64_t& n = P.tile_count[logn];
+    if (n < 0) n = (int64_t)make_tiles(P, int64_t(2) << logn).size();
+    return n;
 }
 
 // Tiles of the batched kernels: every interval on its own.
@@ -355,18 +374,18 @@ static int64_t interval_tiles(const Plan& P, int64_t Lv) {
     return tiles;
 }
 
-// Admissible overlap-save blocks (B = 2^(logn+1) reals > 2 lambda) ordered by the cost
-// model tiles x (N (logn + 1) + 2048) x block weight; the two blocks above the
-// single-CTA maximum run on 2- and 4-CTA clusters.
+// Admissible overlap-save blocks (B = 2^(logn+1) reals > 2 lambda) for R right-hand sides,
+// ordered by modelled time (block_us); the two blocks above the single-CTA maximum run on 2-
+// and 4-CTA clusters.
 template <typename T>
-static std::vector<std::pair<double, int>> block_candidates(const Plan& P) {
+static std::vector<std::pair<double, int>> block_candidates(const Plan& P, int R = 1) {
     const int maxl = toeplitz_max_logn<T>();
     std::vector<std::pair<double, int>> c;
     for (int logn = 8; logn <= maxl + 2; ++logn) {
         const int64_t N = int64_t(1) << logn;
         const int64_t Lv = 2 * N - 2 * (int64_t)P.lambda;
         if (Lv < 1) continue;
-        c.push_back({(double)overlap_tiles(P, Lv) * ((double)N * (logn + 1) + 2048.0) * block_weight<T>(logn), logn});
+        c.push_back({block_us<T>(P, logn, overlap_tiles(P, logn) * R), logn});
     }
     std::stable_sort(c.begin(), c.end());
     return c;
@@ -389,6 +408,22 @@ static int choose_logn(const Plan& P, int forced_log2B, int* cluster) {
     }
     *cluster = logn > maxl ? 1 << (logn - maxl) : 1;
     return logn;
+}
+
+// Overlap-save spectra of the plan's rows for N-point blocks.  The grid of a smaller block is
+// a subset of a larger one's, so the transforms of the largest block asked for so far are kept
+// while the plan is built (three arithmetics ask, often for different blocks).
+static std::vector<std::vector<double>> plan_spectra(Plan& P, int64_t N) {
+    if (P.spec_n < N) {
+        P.spec_n = N;
+        P.spec.clear();
+        for (const auto& r : P.rows) P.spec.push_back(overlap_save_spectrum(r, N));
+    }
+    const int64_t step = P.spec_n / N;
+    std::vector<std::vector<double>> out((size_t)P.npsd, std::vector<double>((size_t)N + 1));
+    for (int p = 0; p < P.npsd; ++p)   // (the spectra are divided by their own N)
+        for (int64_t k = 0; k <= N; ++k) out[(size_t)p][(size_t)k] = P.spec[(size_t)p][(size_t)(k * step)] * (double)step;
+    return out;
 }
 
 template <typename T>
@@ -416,10 +451,10 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
         h2d(tz.ptw, ptT.data(), ptT.size() * sizeof(T), P.stream);
         sync(P.stream);
     }
-    const std::vector<double> Hd = fold_split_spectra(P.rows, N);
+    const std::vector<std::vector<double>> spec = plan_spectra(P, N);
     if constexpr (sizeof(T) == 4) {
         if (tz.cluster == 1 && ws_supported(tz.logn)) {
-            const std::vector<float> tab = ws_tables(tz.logn), Hw = ws_spectra(Hd, P.npsd, tz.logn);
+            const std::vector<float> tab = ws_tables(tz.logn), Hw = ws_spectra(spec, tz.logn);
             tz.ws_tab = dalloc<float>(tab.size());
             h2d(tz.ws_tab, tab.data(), tab.size() * 4, P.stream);
             tz.ws_H = dalloc<float>(Hw.size());
@@ -429,30 +464,36 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
             return;
         }
     }
-    const std::vector<T> H(Hd.begin(), Hd.end());
+    std::vector<T> H;
+    if constexpr (sizeof(T) == 4) {
+        for (const auto& h : spec)
+            for (double v : h) H.push_back((T)(0.25 * v));
+    } else {
+        const std::vector<double> Hd = fold_split_spectra(spec, N);
+        H.assign(Hd.begin(), Hd.end());
+    }
     tz.H = dalloc<T>(H.size());
     h2d(tz.H, H.data(), H.size() * sizeof(T), P.stream);
     sync(P.stream);   // host vectors go out of scope
 }
 
-// Double-float tables on the blocks of the FP64 kernel (tz64, which must be final):
-// its tiles copied, the cosine and per-pass twiddles and the kernel spectra rounded to
-// double-float pairs (hi = FP32 rounding, lo = FP32 rounding of the rest).
-static void build_toeplitz_df(Plan& P) {
-    const ToeplitzDev& src = P.tz64;
+// Double-float tables (where the FP64 kernel has a block): the cosine and per-pass twiddles
+// and the kernel spectra rounded to double-float pairs (hi = FP32 rounding, lo = FP32 rounding
+// of the rest).  The block is the FP64 kernel's where that was asked for, else its own.
+static void build_toeplitz_df(Plan& P, int forced_log2B) {
     ToeplitzDev& tz = P.tzdf;
     free_tz(tz);
     tz = ToeplitzDev{};
-    if (src.logn == 0) return;
-    tz.logn = src.logn;
-    tz.cluster = src.cluster;
-    tz.ntiles = src.ntiles;
+    if (P.tz64.logn == 0) return;
+    tz.logn = choose_logn<dfl>(P, forced_log2B, &tz.cluster);
     const int64_t N = int64_t(1) << tz.logn;
     const int64_t B = 2 * N;
     try {
-        tz.tiles = dalloc<Tile>((size_t)tz.ntiles);
-        check_cuda(cudaMemcpyAsync(tz.tiles, src.tiles, (size_t)tz.ntiles * sizeof(Tile), cudaMemcpyDeviceToDevice,
-                                   P.stream), "copy tiles");
+        const std::vector<Tile> tiles = make_tiles(P, B);
+        tz.ntiles = (int)tiles.size();
+        tz.tiles = dalloc<Tile>(tiles.size());
+        h2d(tz.tiles, tiles.data(), tiles.size() * sizeof(Tile), P.stream);
+        sync(P.stream);
         std::vector<dfl> tw(tz.cluster > 1 ? (size_t)(B / 4 + 1) : 1);
         if (tz.cluster > 1) {   // cross-CTA twiddles
             for (int64_t k = 0; k <= B / 4; ++k) tw[(size_t)k] = dfl(std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B));
@@ -465,7 +506,7 @@ static void build_toeplitz_df(Plan& P) {
         for (size_t i = 0; i < pt.size(); ++i) ptd[i] = dfl(pt[i]);
         tz.ptw = dalloc<dfl>(ptd.size());
         h2d(tz.ptw, ptd.data(), ptd.size() * sizeof(dfl), P.stream);
-        const std::vector<double> Hd = fold_split_spectra(P.rows, N);
+        const std::vector<double> Hd = fold_split_spectra(plan_spectra(P, N), N);
         std::vector<dfl> H(Hd.size());
         for (size_t i = 0; i < Hd.size(); ++i) H[i] = dfl(Hd[i]);
         tz.H = dalloc<dfl>(H.size());
@@ -549,9 +590,11 @@ static void free_sorted_weights(Plan& P) {
 // The sliced layout of the scatter, unless its padding (a slice is as long as its longest
 // pixel, in fours) costs more than half as many entries again: its time is its bytes, the
 // 32-lane form's is about twice that (scatter.cu), so up to there it is ahead.  The FP32
-// I/Q/U scatter of one right-hand side keeps the 32-lane form where that has four or more
-// loads a lane in flight for every pixel (128 samples), pixels enough to fill the chip and a
-// time-domain array that fits the L2 cache: 47.6 us against 52.8 on 65536 pixels of 256.
+// scatter of one right-hand side keeps the 32-lane form while its pixels have 128 to 4095
+// samples (four or more loads a lane in flight, not many in a row) and the time-domain array
+// fits the L2 cache (I/Q/U: 47.6 us against 52.8 on 65536 pixels of 256 samples; T: 26.2
+// against 28.2 on 49000 of 256), and in small I/Q/U plans, where a slice's longer walk shows
+// (5.6 against 7.5 us on 1024 pixels of 256).
 static void build_sliced(Plan& P) {
     constexpr int PIX = 8;
     if (P.npix_obs == 0) return;
@@ -569,7 +612,8 @@ static void build_sliced(Plan& P) {
     }
     P.sl_count = ns;
     P.sl_steps = steps;
-    P.sl_f32 = P.ncomp == 1 || P.nkept < (int64_t)128 * P.npix_obs || P.npix_obs < P.num_sms * 64 || P.nt > (1 << 25);
+    const int64_t hits = P.nkept / P.npix_obs;
+    P.sl_f32 = hits >= 4096 || P.nt > (1 << 25) || (hits < 128 && P.nkept >= (1 << 20)) || (P.ncomp == 1 && P.nkept < (1 << 20));
     const size_t e = (size_t)steps * 32 + SL_PAD;
     try {
         P.sl_off = dalloc<int32_t>(off.size());
@@ -763,6 +807,18 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
     h2d(P.ipsd, P.h_ipsd.data(), (size_t)K * 4, s);
     P.t0 = dalloc<double>((size_t)npsd);
     h2d(P.t0, t0.data(), (size_t)npsd * 8, s);
+    {   // the largest block first: its spectra serve the others
+        int cl, logn = 0;
+        for (int k = 0; k < 3; ++k) {
+            try {
+                logn = std::max(logn, k == 0   ? choose_logn<double>(P, o->fft_log2_f64, &cl)
+                                      : k == 1 ? choose_logn<float>(P, o->fft_log2_f32, &cl)
+                                               : choose_logn<dfl>(P, o->fft_log2_f64, &cl));
+            } catch (const Error&) {   // reported by the build below
+            }
+        }
+        if (logn > 0) (void)plan_spectra(P, int64_t(1) << logn);
+    }
     // A precision whose largest block cannot hold the band is left unbuilt (logn = 0):
     // its operators then fail with MM_ERR_ARG; at least one precision must exist.
     for (int prec = 0; prec < 2; ++prec) {
@@ -811,6 +867,7 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
     check_cuda(cudaEventCreate(&P.ev1), "event");
     check_cuda(cudaEventCreate(&P.ev2), "event");
     P.autotune = o->autotune != 0;
+    P.forced_f32 = o->fft_log2_f32 > 0;
     if (o->scatter_lanes != 0) {
         if (o->scatter_lanes != 32 && o->scatter_lanes != 16 && o->scatter_lanes != 8)
             throw Error{MM_ERR_ARG, "scatter_lanes must be 0, 32, 16 or 8"};
@@ -845,7 +902,9 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
         }
     }
     free_sorted_weights(P);
-    build_toeplitz_df(P);
+    build_toeplitz_df(P, o->fft_log2_f64);
+    P.spec.clear();
+    P.spec_n = 0;
     sync(s);
 }
 
@@ -1641,7 +1700,9 @@ static void ensure_grad(PlanHolder& P) {
                                                 P.h_psd[(size_t)p].alpha, P.L_grid, P.fsamp, P.lambda, P.window);
         for (int c = 0; c < 3; ++c) rows[(size_t)c * P.npsd + p] = D[(size_t)c];
     }
-    const std::vector<double> H = fold_split_spectra(rows, N);
+    std::vector<std::vector<double>> spec;
+    for (const auto& r : rows) spec.push_back(overlap_save_spectrum(r, N));
+    const std::vector<double> H = fold_split_spectra(spec, N);
     P.grad_H = dalloc<double>(H.size());
     h2d(P.grad_H, H.data(), H.size() * 8, P.stream);
     P.grad_u = dalloc<double>((size_t)P.nt);
@@ -1832,7 +1893,7 @@ static void ensure_batch_tc_buffer(PlanHolder& P, int R) {
 }
 
 static void launch_batch_tz(PlanHolder& P, int R, const float* X, float* Z, const int* done);
-static void launch_batch_tz(PlanHolder& P, int R, const float* X, float* Z, const int* done);
+static const ToeplitzDev& batch_tz(const PlanHolder& P) { return P.batch.tz.logn != 0 ? P.batch.tz : P.tz32; }
 
 // Batched Toeplitz form, chosen once per plan (before any graph capture), after the
 // R-column buffers exist:
@@ -1840,8 +1901,8 @@ static void launch_batch_tz(PlanHolder& P, int R, const float* X, float* Z, cons
 //               block > 2 lambda complex points);
 //   BATCH_REAL  the single-RHS real-FFT kernel with an RHS grid dimension (its FP32
 //               block, B > 2 lambda reals, so half the FFT length of the pair form).
-// Cost model per RHS: tiles x (points x log2 + 2048) x cluster weight, halved for the
-// pair form; ties go to the pair form.  With autotuning both are timed at this R.
+// Cost model: block_us of the real form's tiles, and for the pair form its operation count at
+// a measured rate; ties go to the pair form.  With autotuning both are timed at this R.
 static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
     BatchState& bt = P.batch;
     if (bt.kind >= 0) {
@@ -1862,16 +1923,35 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
         const int64_t Lv = B - 2 * (int64_t)P.lambda;
         if (Lv < 1) continue;
         const int cl = logb > BATCH_MAX_LOGB_CTA ? 1 << (logb - BATCH_MAX_LOGB_CTA) : 1;
-        const double cost = 0.5 * (double)interval_tiles(P, Lv) * ((double)B * logb + 2048.0) * fp32_cluster_weight(cl);
+        // two right-hand sides per transform; SM time per operation measured at lambda = 1024
+        // .. 16384, the cluster blocks' relative to it
+        const double weight = cl == 4 ? 3.3 : (cl == 2 ? 1.6 : 1.0);
+        const double us = (double)interval_tiles(P, Lv) * ((R + 1) / 2) * ((double)B * logb + 2048.0) * weight * 1.28e-4;
+        const double cost = std::max(15.0, us / P.num_sms);
         if (best < 0 || cost < best_cost) {
             best = logb;
             best_cost = cost;
         }
     }
+    // the real form's block for this many right-hand sides: one that fills the chip with R
+    // launches' worth of tiles can be larger than the one with the shortest single launch
     double real_cost = -1.0;
     if (P.tz32.logn != 0) {
-        const int64_t N = int64_t(1) << P.tz32.logn;
-        real_cost = (double)P.tz32.ntiles * ((double)N * (P.tz32.logn + 1) + 2048.0) * block_weight<float>(P.tz32.logn);
+        int logn = P.tz32.logn;
+        real_cost = block_us<float>(P, logn, (int64_t)P.tz32.ntiles * R);
+        if (!P.forced_f32 && !P.autotune) {
+            const auto c = block_candidates<float>(P, R);
+            if (c[0].first < 0.95 * real_cost) {
+                logn = c[0].second;
+                real_cost = c[0].first;
+            }
+        }
+        if (logn != P.tz32.logn && want != BATCH_PAIR && (want == BATCH_REAL || best < 0 || real_cost < best_cost))
+        {
+            build_toeplitz<float>(P, bt.tz, logn + 1);
+            P.spec.clear();
+            P.spec_n = 0;
+        }
     }
     if (best < 0 && real_cost < 0.0) throw Error{MM_ERR_ARG, "lambda too large for the batched FFT blocks"};
     if ((want == BATCH_PAIR && best < 0) || (want == BATCH_REAL && real_cost < 0.0))
@@ -1964,7 +2044,7 @@ static BatchTzArgs batch_tz_args(PlanHolder& P, int R, const float* X, float* Z,
 static void launch_batch_tz(PlanHolder& P, int R, const float* X, float* Z, const int* done) {
     BatchState& bt = P.batch;
     if (bt.kind == BATCH_REAL) {
-        launch_toeplitz_rhs<float>(P, P.tz32, nullptr, X, R, P.n, Z, P.nt, done, P.stream);
+        launch_toeplitz_rhs<float>(P, batch_tz(P), nullptr, X, R, P.n, Z, P.nt, done, P.stream);
     } else if (bt.kind == BATCH_TENSOR) {
         // column scales from the maps, Y = P X, then the band product on the tensor cores
         launch_batch_colscale(X, P.n, R, bt.tc_scale, bt.tc_scale + BATCH_RMAX, P.stream);
@@ -2118,7 +2198,7 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
         // b_r = P^T N^-1 d_r in FP32 for all columns in one batched Toeplitz launch (it seeds
         // the first inner solve and scales the residual; the FP64 residuals come from the
         // data, residual64)
-        launch_toeplitz_any<float>(P, P.tz32, nullptr, Dg, nullptr, Rc, (int64_t)nt, bt.tod, (int64_t)nt, nullptr, s);
+        launch_toeplitz_any<float>(P, batch_tz(P), nullptr, Dg, nullptr, Rc, (int64_t)nt, bt.tod, (int64_t)nt, nullptr, s);
         launch_batch_scatter(P, bt.tod, bt.z, Rc, nullptr, s);
         launch_convert_f32_to_f64(bt.z, bt.b64, (int64_t)Rc * n, s);
         for (int r = 0; r < Rc; ++r) {
@@ -2594,7 +2674,7 @@ mm_status mm_batch_config(mm_plan_t plan, int32_t R, int32_t* kind, int32_t* log
         sync(*P);
         const BatchState& bt = P->batch;
         *kind = bt.kind;
-        if (log2_block) *log2_block = bt.kind == BATCH_REAL ? P->tz32.logn + 1 : (bt.kind == BATCH_TENSOR ? 7 : bt.logb);
+        if (log2_block) *log2_block = bt.kind == BATCH_REAL ? batch_tz(*P).logn + 1 : (bt.kind == BATCH_TENSOR ? 7 : bt.logb);
         if (ms) {
             ms[0] = bt.tuned_ms[0];
             ms[1] = bt.tuned_ms[1];

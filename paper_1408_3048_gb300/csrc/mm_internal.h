@@ -64,7 +64,8 @@ struct ToeplitzDev {
     void* ws_tab = nullptr;
     void* ws_H = nullptr;
     float* ws_scratch = nullptr;
-    void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N, folded (fold_split_spectra)
+    void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N, folded (fold_split_spectra);
+                             // FP32: T[npsd][N + 1], divided by another 4 (split_chain)
 };
 
 struct CoarseDev {
@@ -165,7 +166,10 @@ struct Plan {
     double* t0 = nullptr;          // [npsd] diagonal of each row
 
     ToeplitzDev tz64, tz32;
-    ToeplitzDev tzdf;              // double-float tables on tz64's blocks (refinement residual)
+    ToeplitzDev tzdf;              // double-float tables (refinement residual)
+    std::vector<std::vector<double>> spec;   // spectra of the rows while tables are built (N = spec_n)
+    int64_t spec_n = 0;
+    mutable int64_t tile_count[20] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
 
     // block-Jacobi: inverse blocks, symmetric packed (a00 a01 a02 a11 a12 a22) or 1
     double* bd64 = nullptr;        // [npix_obs][ncomp == 3 ? 6 : 1]
@@ -251,7 +255,7 @@ std::vector<std::vector<double>> toeplitz_row_derivatives(double sigma, double f
 std::vector<double> overlap_save_spectrum(const std::vector<double>& t, int64_t N);
 // values of a folded spectrum: alpha [N], beta [N/2 + 1], one of padding
 __host__ __device__ constexpr int64_t split_size(int64_t N) { return N + N / 2 + 2; }
-std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& rows, int64_t N);
+std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& spectra, int64_t N);
 // per-pass Stockham twiddles of an N = 2^logn point FFT as interleaved (cos, sin)
 std::vector<double> pass_twiddle_table(int logn);
 double rcond_sym3(const double B[6]);
@@ -281,7 +285,7 @@ void launch_toeplitz_f32_packed(const Plan& P, const float* x, bool pack, float*
                                 cudaStream_t s);
 bool ws_supported(int logn);
 std::vector<float> ws_tables(int logn);
-std::vector<float> ws_spectra(const std::vector<double>& folded, int npsd, int logn);
+std::vector<float> ws_spectra(const std::vector<std::vector<double>>& spectra, int logn);
 size_t ws_scratch_floats(int logn, int num_sms);
 template <typename T>
 size_t toeplitz_smem_bytes(int logn);

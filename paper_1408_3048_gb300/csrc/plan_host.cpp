@@ -152,12 +152,12 @@ std::vector<double> overlap_save_spectrum(const std::vector<double>& t, int64_t 
     return h;
 }
 
-// Overlap-save spectra h (k = 0..N, over 2N points) of kernel rows, folded for the product of
+// Overlap-save spectra h (k = 0..N, over 2N points; overlap_save_spectrum) folded for the product of
 // a packed real block (toeplitz.cuh, split_product): with W = exp(-i pi k / N) = c - i s,
 // hs = (h_k + h_{N-k}) / 2 and hd = (h_k - h_{N-k}) / 2,
 //   alpha_k = hs - s hd  (k = 0..N-1),   beta_k = c hd  (k = 0..N/2; beta_{N-k} = beta_k),
 // per row alpha first, then beta, split_size(N) values (the last is padding).
-std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& rows, int64_t N) {
+std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& spectra, int64_t N) {
     const int64_t hs = split_size(N);
     std::vector<double> sn((size_t)(N / 2 + 1)), cs((size_t)(N / 2 + 1));   // sin is even about N / 2
     for (int64_t k = 0; k <= N / 2; ++k) {
@@ -165,9 +165,9 @@ std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& r
         sn[(size_t)k] = std::sin(th);
         cs[(size_t)k] = std::cos(th);
     }
-    std::vector<double> f((size_t)((int64_t)rows.size() * hs), 0.0);
-    for (size_t p = 0; p < rows.size(); ++p) {
-        const std::vector<double> h = overlap_save_spectrum(rows[p], N);
+    std::vector<double> f((size_t)((int64_t)spectra.size() * hs), 0.0);
+    for (size_t p = 0; p < spectra.size(); ++p) {
+        const std::vector<double>& h = spectra[p];
         double* al = f.data() + (int64_t)p * hs;
         for (int64_t k = 0; k < N; ++k) {
             const double sum = 0.5 * (h[(size_t)k] + h[(size_t)(N - k)]);

@@ -69,7 +69,7 @@ struct TzArgs {
     const Tile* tiles;
     const T* twiddle;      // [N/2 + 1]: cos(2 pi k / B), cross-CTA step of the cluster blocks
     const typename Cx<T>::type* ptw;  // per-pass FFT twiddles (ptw_offset)
-    const T* H;            // [npsd][split_size(N)] folded spectra
+    const T* H;            // [npsd][split_size(N)] folded spectra; FP32: [npsd][N + 1] spectra / 4
     const In<T>* y;        // time-domain input (mode 0)
     const double* yd;      // FP64 time-domain input (modes 2, 4, 5)
     const In<T>* x;        // map (gather modes)
@@ -616,15 +616,15 @@ __device__ __forceinline__ void store_out(const Tile& tile, In<T>* z, int lambda
     if (in) z[p + seg_d(tile, g)] = to_in<T>(v);
 }
 
-// Spectrum product of the packed real block at the bin pair (k, N - k).  Written out, the
-// chain real-FFT split -> product with the real kernel spectrum -> merge back to packed form
-// is linear in u1 = U_k and conj(u2), u2 = U_{N-k}, with real coefficients that depend on the
-// kernel and k alone (fold_split_spectra):
+// Spectrum product of the packed real block at the bin pair (k, N - k), u1 = U_k, u2 =
+// U_{N-k}, returned conjugated: the forward FFT of conj(V) is conj of N * IFFT(V).
+//
+// FP64 and double-float: written out, the chain real-FFT split -> product with the real kernel
+// spectrum -> merge back to packed form is linear in u1 and conj(u2) with real coefficients
+// that depend on the kernel and k alone (fold_split_spectra):
 //   V_k = alpha_k u1 + i beta_k conj(u2),   V_{N-k} = alpha_{N-k} u2 + i beta_k conj(u1),
-// eight operations for the pair and no twiddle, where the chain done step by step took 44
-// and a sine and cosine per pair (one A x in FP64 on 2^22 samples at lambda = 4096: 1.003 ->
-// 0.924 ms, FP64-pipe bound; FP32 on 2^24: 219 -> 213 us).  Returned conjugated: the forward FFT of conj(V) is conj of
-// N * IFFT(V).
+// eight operations for the pair and no twiddle, where the chain took 44 (one A x in FP64 on
+// 2^22 samples at lambda = 4096: 1.003 -> 0.924 ms, FP64-pipe bound).
 template <typename T>
 __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename Cx<T>::type u2, T a1, T a2, T b,
                                               typename Cx<T>::type& V1, typename Cx<T>::type& V2) {
@@ -632,6 +632,28 @@ __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename 
     V1.y = -(a1 * u1.y + b * u2.x);
     V2.x = a2 * u2.x + b * u1.y;
     V2.y = -(a2 * u2.y + b * u1.x);
+}
+
+// FP32: the chain itself.  1/f noise leaves H_k small at the low bins, where a map's time
+// stream is largest; the chain multiplies the rounding errors of X_k by H_k, the folded form
+// leaves them at full size in both bins of the pair.  The error against 64 bits is the same
+// in norm, but it sits in the slow modes: FP32 PCG runs took 10 % more iterations on it.
+// h1 = H_k / 4, h2 = H_{N-k} / 4, (cw, sw) = (cos, sin) of pi k / N.
+__device__ __forceinline__ void split_chain(float2 u1, float2 u2, float cw, float sw, float h1, float h2, float2& V1,
+                                            float2& V2) {
+    // twice E = (u1 + conj u2) / 2 and O = -i (u1 - conj u2) / 2
+    const float2 E = make_float2(u1.x + u2.x, u1.y - u2.y);
+    const float2 O = make_float2(u1.y + u2.y, u2.x - u1.x);
+    const float2 WO = cmul<float>(O, cw, sw);
+    // X_k = E + W O, conj X_{N-k} = E - W O, times the spectrum
+    const float2 Z1 = make_float2(h1 * (E.x + WO.x), h1 * (E.y + WO.y));
+    const float2 Z2 = make_float2(h2 * (E.x - WO.x), h2 * (E.y - WO.y));
+    // V_k = S + i conj(W) D, conj V_{N-k} = S - i conj(W) D
+    const float2 S = make_float2(Z1.x + Z2.x, Z1.y + Z2.y);
+    const float2 D = make_float2(Z1.x - Z2.x, Z1.y - Z2.y);
+    const float px = cw * D.x - sw * D.y, py = cw * D.y + sw * D.x;
+    V1 = make_float2(S.x - py, -(S.y + px));
+    V2 = make_float2(S.x + py, S.y - px);
 }
 
 template <typename T, int LOGN, int NT, int MODE>
@@ -654,15 +676,43 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
     __syncthreads();
     prefetch_issue<T, MODE>(A, next);
     fft_all<T, LOGN, NT, 0>(a, A.ptw);
-    constexpr int64_t HS = split_size(N);
-    const T* al = A.H + tile.psd * HS;
-    const T* be = al + N;
-    for (int k = tid; k <= N / 2; k += NT) {
-        const int k2 = (N - k) & (N - 1);
-        C2 V1, V2;
-        split_product<T>(a[pad<T>(k)], a[pad<T>(k2)], al[k], al[k2], be[k], V1, V2);
-        a[pad<T>(k)] = V1;
-        if (k2 != k) a[pad<T>(k2)] = V2;
+    if constexpr (sizeof(T) == 4) {
+        // spectrum values of U bin pairs are requested together; bin N/2, its own partner, apart
+        const T* H = A.H + (int64_t)tile.psd * (N + 1);
+        constexpr int PER = N / 2 / NT, U = PER < 8 ? PER : 8;
+        auto product = [&](int k, T h1, T h2) {
+            const int k2 = (N - k) & (N - 1);
+            float sw, cw;
+            sincospif((float)k * (1.f / (float)N), &sw, &cw);
+            C2 V1, V2;
+            split_chain(a[pad<T>(k)], a[pad<T>(k2)], cw, sw, h1, h2, V1, V2);
+            a[pad<T>(k)] = V1;
+            if (k2 != k) a[pad<T>(k2)] = V2;
+        };
+#pragma unroll 1
+        for (int h = 0; h < PER; h += U) {
+            T h1[U], h2[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int k = tid + (h + u) * NT;
+                h1[u] = __ldg(H + k);
+                h2[u] = __ldg(H + N - k);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) product(tid + (h + u) * NT, h1[u], h2[u]);
+        }
+        if (tid == 0) product(N / 2, __ldg(H + N / 2), __ldg(H + N / 2));
+    } else {
+        constexpr int64_t HS = split_size(N);
+        const T* al = A.H + tile.psd * HS;
+        const T* be = al + N;
+        for (int k = tid; k <= N / 2; k += NT) {
+            const int k2 = (N - k) & (N - 1);
+            C2 V1, V2;
+            split_product<T>(a[pad<T>(k)], a[pad<T>(k2)], al[k], al[k2], be[k], V1, V2);
+            a[pad<T>(k)] = V1;
+            if (k2 != k) a[pad<T>(k2)] = V2;
+        }
     }
     __syncthreads();
     fft_all<T, LOGN, NT, 0>(a, A.ptw);
@@ -781,9 +831,21 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     for (int u = 0; u < PER; ++u) a[pad<T>(u * NT + tid)] = y[u];
     __syncthreads();
     fft_all<T, LOGM, NT, 0>(a, A.ptw);
-    constexpr int64_t HS = split_size(N);
+    constexpr bool F32 = sizeof(T) == 4;
+    constexpr int64_t HS = F32 ? N + 1 : split_size(N);
     const T* al = A.H + tile.psd * HS;
     const T* be = al + N;
+    // bins k and N - k (FP32: the chain, al = the spectrum itself)
+    auto product = [&](C2 u1, C2 u2, int k, C2& V1, C2& V2) {
+        const int k2 = (N - k) & (N - 1);
+        if constexpr (F32) {
+            T cw, sw;
+            twiddle<T, LOGQ>(A.twiddle, k, cw, sw);
+            split_chain(u1, u2, cw, sw, al[k], al[N - k], V1, V2);
+        } else {
+            split_product<T>(u1, u2, al[k], al[k2], be[k < k2 ? k : k2], V1, V2);
+        }
+    };
     const int prank = (CL - rank) % CL;
     if (prank == rank) {
         // partner bins inside this CTA: process each pair once
@@ -791,9 +853,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
         for (int k1 = tid; k1 < npairs; k1 += NT) {
             const int k = CL * k1 + rank;
             const int p = rank == 0 ? ((M - k1) & (M - 1)) : (M - 1 - k1);
-            const int k2 = (N - k) & (N - 1);
             C2 V1, V2;
-            split_product<T>(a[pad<T>(k1)], a[pad<T>(p)], al[k], al[k2], be[k < k2 ? k : k2], V1, V2);
+            product(a[pad<T>(k1)], a[pad<T>(p)], k, V1, V2);
             a[pad<T>(k1)] = V1;
             if (p != k1) a[pad<T>(p)] = V2;
         }
@@ -808,8 +869,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
             const int k1 = u * NT + tid;
             const int k = CL * k1 + rank;
             C2 V2;
-            split_product<T>(a[pad<T>(k1)], part[prank][pad<T>(M - 1 - k1)], al[k], al[N - k],
-                             be[k < N - k ? k : N - k], vo[u], V2);
+            product(a[pad<T>(k1)], part[prank][pad<T>(M - 1 - k1)], k, vo[u], V2);
         }
         cl.sync();
 #pragma unroll

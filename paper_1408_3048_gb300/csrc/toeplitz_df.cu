@@ -1,7 +1,7 @@
 // Double-float instantiations of the overlap-save Toeplitz kernel (see toeplitz.cuh and
 // dfloat.cuh): N^-1 of Eq. 4 on FP64 data with the FFT in double-float arithmetic on the
 // FP32 pipe, for the refinement residual P^T N^-1 (d - P x) of the mixed solver (Eq. 5,
-// 7).  Same blocks, tiles and thread counts as the FP64 kernel.
+// 7).  Same blocks and thread counts as the FP64 kernel.
 #include "toeplitz.cuh"
 
 namespace mm {
@@ -19,6 +19,9 @@ static void df_single(const TzArgs<dfl>& A, int ntiles, int mode, cudaStream_t s
     if (mode == 5) return launch_one<dfl, LOGN, 5>(A, ntiles, s);
     throw Error{MM_ERR_ARG, "unsupported double-float Toeplitz load mode"};
 }
+
+template <>
+int toeplitz_max_logn<dfl>() { return 13; }
 
 void launch_toeplitz_df(const Plan& P, const double* y, const double* d, const double* x, int R, int64_t in_stride,
                         double* z, int64_t out_stride, cudaStream_t s) {

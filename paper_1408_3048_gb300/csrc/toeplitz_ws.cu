@@ -47,7 +47,8 @@ constexpr int WS_REG_FFT = 88, WS_REG_GATHER = 40;
 // (c, c, s, s) for forward pass 2, whose two butterflies share a class, and (c, c', s, s') of
 // two neighbouring positions for the inverse passes; (c, s) of t and t^4 for forward pass 3.
 // Behind them, in global memory only: (t, t^4) of two neighbouring positions for the last
-// pass, by thread, and t of the middle pass's tasks (float2).
+// pass, by thread, and t and its square root, the split's
+// twiddle, of the middle pass's tasks.
 template <int LOGN>
 struct WsTab {
     static constexpr int N = 1 << LOGN;
@@ -123,39 +124,36 @@ std::vector<float> ws_tables(int logn) {
         int p, pm;
         ws_task_host(task, p, pm);
         one(-(double)brv(p, 12) / N);
+        one(-0.5 * (double)brv(p, 12) / N);
     }
     return out;
 }
 
-// Folded spectra (fold_split_spectra) in the order of the middle pass, per PSD: three arrays
-// [WS_TASKS][RM] -- alpha of bin k0 + 4096 s of the first sub-block, alpha of its partner bin
-// in the second, beta of that pair -- then [RM] beta of sub-block 1 (task 0).
-int64_t ws_spectrum_size(int logn) { return (int64_t)(3 * WS_TASKS + 1) * ((1 << logn) / 4096); }
+// Spectra / 4 (split_chain) in the order of the middle pass, per PSD: two arrays
+// [WS_TASKS][RM], of the bins k0 + 4096 s of a task's first sub-block and of their partners
+// N - k; then [RM], the first RM / 2 bins of sub-block 1 (task 0) and their partners.
+int64_t ws_spectrum_size(int logn) { return (int64_t)(2 * WS_TASKS + 1) * ((1 << logn) / 4096); }
 
-std::vector<float> ws_spectra(const std::vector<double>& folded, int npsd, int logn) {
+std::vector<float> ws_spectra(const std::vector<std::vector<double>>& spectra, int logn) {
     const int N = 1 << logn, RM = N / 4096;
-    const int64_t hs = split_size(N), sz = ws_spectrum_size(logn), part = (int64_t)WS_TASKS * RM;
-    std::vector<float> out((size_t)(npsd * sz), 0.f);
-    std::vector<int> k0((size_t)2 * WS_TASKS);
-    for (int task = 0; task < WS_TASKS; ++task) {
-        int p, pm;
-        ws_task_host(task, p, pm);
-        k0[(size_t)2 * task] = brv(p, 12);
-        k0[(size_t)2 * task + 1] = brv(pm, 12);
-    }
-    for (int q = 0; q < npsd; ++q) {
-        const double* al = folded.data() + q * hs;
-        const double* be = al + N;
-        float* o = out.data() + q * sz;
-        auto beta = [&](int k) { return (float)be[k <= N / 2 ? k : N - k]; };
-        for (int task = 0; task < WS_TASKS; ++task)
+    const int64_t sz = ws_spectrum_size(logn), part = (int64_t)WS_TASKS * RM;
+    std::vector<float> out(spectra.size() * (size_t)sz, 0.f);
+    for (size_t q = 0; q < spectra.size(); ++q) {
+        const std::vector<double>& h = spectra[q];
+        float* o = out.data() + q * (size_t)sz;
+        for (int task = 0; task < WS_TASKS; ++task) {
+            int p, pm;
+            ws_task_host(task, p, pm);
+            const int k0 = brv(p, 12);
             for (int e = 0; e < RM; ++e) {
-                const int a = k0[(size_t)2 * task] + 4096 * e, b = k0[(size_t)2 * task + 1] + 4096 * (RM - 1 - e);
-                o[(int64_t)task * RM + e] = (float)al[a];
-                o[part + (int64_t)task * RM + e] = (float)al[b];
-                o[2 * part + (int64_t)task * RM + e] = beta(a);
+                o[(int64_t)task * RM + e] = (float)(0.25 * h[(size_t)(k0 + 4096 * e)]);
+                o[part + (int64_t)task * RM + e] = (float)(0.25 * h[(size_t)(N - k0 - 4096 * e)]);
             }
-        for (int e = 0; e < RM; ++e) o[3 * part + e] = beta(2048 + 4096 * e);
+        }
+        for (int e = 0; e < RM / 2; ++e) {
+            o[2 * part + e] = (float)(0.25 * h[(size_t)(2048 + 4096 * e)]);
+            o[2 * part + RM / 2 + e] = (float)(0.25 * h[(size_t)(N - 2048 - 4096 * e)]);
+        }
     }
     return out;
 }
@@ -286,17 +284,6 @@ __device__ __forceinline__ void scale_powers(cx2* v, cx2 t, cx2 t4) {
         if (a == 1) W = mul2(t4, t4);
         if (a == 2) W = mul2(t4, W);
     }
-}
-
-// V1 = a1 u1 + i b conj(u2), V2 = a2 u2 + i b conj(u1) in place
-__device__ __forceinline__ void ws_pair(float2& u1, float2& u2, float a1, float a2, float b) {
-    float2 V1, V2;
-    V1.x = fmaf(a1, u1.x, b * u2.y);
-    V1.y = fmaf(a1, u1.y, b * u2.x);
-    V2.x = fmaf(a2, u2.x, b * u1.y);
-    V2.y = fmaf(a2, u2.y, b * u1.x);
-    u1 = V1;
-    u2 = V2;
 }
 
 __host__ __device__ constexpr int brv4(int r) { return ((r & 1) << 3) | ((r & 2) << 1) | ((r & 4) >> 1) | ((r & 8) >> 3); }
@@ -541,10 +528,32 @@ __device__ __forceinline__ void dftm(float2* v) {
     else bfly2<float>(v[0], v[1]);
 }
 
+// split_chain (toeplitz.cuh) for two bin pairs at a time, V unconjugated: w = exp(-i pi k / N)
+__device__ __forceinline__ void chain2(cx2& u1, cx2& u2, cx2 w, f2 h1, f2 h2) {
+    const cx2 E = {add2(u1.re, u2.re), sub2(u1.im, u2.im)};
+    const cx2 F = {sub2(u1.re, u2.re), add2(u1.im, u2.im)};   // O = -i F
+    const cx2 WO = {fma2(w.re, F.im, mul2(w.im, F.re)), sub2(mul2(w.im, F.im), mul2(w.re, F.re))};
+    const cx2 Z1 = {mul2(h1, add2(E.re, WO.re)), mul2(h1, add2(E.im, WO.im))};
+    const cx2 Z2 = {mul2(h2, sub2(E.re, WO.re)), mul2(h2, sub2(E.im, WO.im))};
+    const cx2 S = add2(Z1, Z2), D = sub2(Z1, Z2);
+    const cx2 P = {fma2(w.re, D.re, mul2(w.im, D.im)), sub2(mul2(w.re, D.im), mul2(w.im, D.re))};   // conj(W) D
+    u1 = {sub2(S.re, P.im), add2(S.im, P.re)};
+    u2 = {add2(S.re, P.im), sub2(P.re, S.im)};
+}
+
+// the same for one pair
+__device__ __forceinline__ void chain1(float2& u1, float2& u2, float2 w, float h1, float h2) {
+    float2 V1, V2;
+    split_chain(u1, u2, w.x, -w.y, h1, h2, V1, V2);
+    u1 = make_float2(V1.x, -V1.y);
+    u2 = make_float2(V2.x, -V2.y);
+}
+
 // Sub-blocks sa and sb of one task: last forward radix, product, first inverse radix.
+// tw = (t, exp(-i pi k0 / N)).
 template <int RM, int PLANE>
-__device__ __forceinline__ void ws_middle(float* sa, float* sb, float2 t, const float (&a1)[RM], const float (&a2)[RM],
-                                          const float (&be)[RM], bool self, const float* __restrict__ b1) {
+__device__ __forceinline__ void ws_middle(float* sa, float* sb, float4 tw, const float (&h1)[RM], const float (&h2)[RM],
+                                          bool self, const float* __restrict__ b1) {
     float2 va[RM], vb[RM];
 #pragma unroll
     for (int r = 0; r < RM; r += 2) {
@@ -555,6 +564,7 @@ __device__ __forceinline__ void ws_middle(float* sa, float* sb, float2 t, const 
         vb[r] = make_float2(xb.x, yb.x);
         vb[r + 1] = make_float2(xb.y, yb.y);
     }
+    const float2 t = make_float2(tw.x, tw.y);
     // the second sub-block's root is exp(-2 pi i (4096 - k0) / N) = exp(-2 pi i / RM) conj(t)
     // (task 0: exp(-2 pi i 2048 / N) instead, t = 1 for the first)
     float2 u = RM == 4 ? make_float2(-t.y, -t.x) : make_float2(-t.x, t.y);
@@ -570,20 +580,38 @@ __device__ __forceinline__ void ws_middle(float* sa, float* sb, float2 t, const 
     }
     dftm<RM>(va);
     dftm<RM>(vb);
+    // twiddle of bin k0 + 4096 s: exp(-i pi k0 / N) times exp(-i pi s / RM)
     if (!self) {
+        const float2 w0 = make_float2(tw.z, tw.w);
+        float2 w1 = RM == 4 ? mulc(w0, make_float2(WS_H, -WS_H)) : make_float2(w0.y, -w0.x);
+        cx2 w = {pk(w0.x, w1.x), pk(w0.y, w1.y)};
 #pragma unroll
-        for (int s = 0; s < RM; ++s) ws_pair(va[s], vb[RM - 1 - s], a1[s], a2[s], be[s]);
+        for (int s = 0; s < RM; s += 2) {
+            const int m = RM - 1 - s;
+            cx2 a = {pk(va[s].x, va[s + 1].x), pk(va[s].y, va[s + 1].y)};
+            cx2 b = {pk(vb[m].x, vb[m - 1].x), pk(vb[m].y, vb[m - 1].y)};
+            if (s == 2) w = {pk(w0.y, w1.y), pk(-w0.x, -w1.x)};   // times -i
+            chain2(a, b, w, pk(h1[s], h1[s + 1]), pk(h2[s], h2[s + 1]));
+            const float2 ar = upk(a.re), ai = upk(a.im), br = upk(b.re), bi = upk(b.im);
+            va[s] = make_float2(ar.x, ai.x);
+            va[s + 1] = make_float2(ar.y, ai.y);
+            vb[m] = make_float2(br.x, bi.x);
+            vb[m - 1] = make_float2(br.y, bi.y);
+        }
     } else {
         // k0 = 0: bins 0 and N/2 are their own partners, else s and RM - s; k0 = 2048: s and
         // RM - 1 - s
-#pragma unroll
-        for (int s = 0; s < RM; s += RM / 2) {
-            const float2 x = va[s];
-            va[s] = make_float2(fmaf(a1[s], x.x, be[s] * x.y), fmaf(a1[s], x.y, be[s] * x.x));
+        float2 x = va[0];
+        chain1(va[0], x, make_float2(1.f, 0.f), h1[0], h2[0]);
+        x = va[RM / 2];
+        chain1(va[RM / 2], x, make_float2(0.f, -1.f), h1[RM / 2], h2[RM / 2]);
+        if constexpr (RM == 4) {
+            chain1(va[1], va[3], make_float2(WS_H, -WS_H), h1[1], h2[1]);
+            chain1(vb[0], vb[3], make_float2(WS_C1, -WS_S1), __ldg(b1), __ldg(b1 + 2));
+            chain1(vb[1], vb[2], make_float2(WS_S1, -WS_C1), __ldg(b1 + 1), __ldg(b1 + 3));
+        } else {
+            chain1(vb[0], vb[1], make_float2(WS_H, -WS_H), __ldg(b1), __ldg(b1 + 1));
         }
-        if constexpr (RM == 4) ws_pair(va[1], va[3], a1[1], a1[3], be[1]);
-#pragma unroll
-        for (int s = 0; s < RM / 2; ++s) ws_pair(vb[s], vb[RM - 1 - s], a2[RM - 1 - s], a2[s], __ldg(b1 + s));
     }
 #pragma unroll
     for (int s = 0; s < RM; ++s) {
@@ -637,34 +665,30 @@ __device__ __forceinline__ void ws_transform(const TzArgs<float>& A, const Tile*
     // middle: the spectrum values of a task are requested one task ahead
     {
         constexpr int TPT = WS_TASKS / NF;
-        const float* H = Hall + tp->psd * ((int64_t)(3 * WS_TASKS + 1) * RM);
-        const float2* mt = reinterpret_cast<const float2*>(gtab + TB::MT);
+        const float* H = Hall + tp->psd * ((int64_t)(2 * WS_TASKS + 1) * RM);
+        const float4* mt = gtab + TB::MT;
         int task = warp * (32 * TPT) + (tid & 31);
-        float a1[RM], a2[RM], be[RM];
-        ldn<RM>(a1, H + task * RM);
-        ldn<RM>(a2, H + (WS_TASKS + task) * RM);
-        ldn<RM>(be, H + (2 * WS_TASKS + task) * RM);
-        float2 t = __ldg(mt + task);
+        float h1[RM], h2[RM];
+        ldn<RM>(h1, H + task * RM);
+        ldn<RM>(h2, H + (WS_TASKS + task) * RM);
+        float4 t = __ldg(mt + task);
         group_sync(warp);
 #pragma unroll 1
         for (int i = 0; i < TPT; ++i) {
-            float n1[RM], n2[RM], nb[RM];
-            float2 nt;
+            float n1[RM], n2[RM];
+            float4 nt;
             if (i + 1 < TPT) {
                 ldn<RM>(n1, H + (task + 32) * RM);
                 ldn<RM>(n2, H + (WS_TASKS + task + 32) * RM);
-                ldn<RM>(nb, H + (2 * WS_TASKS + task + 32) * RM);
                 nt = __ldg(mt + task + 32);
             }
             int p, pm;
             ws_task(task, task == 0 ? 0 : 1 << (31 - __clz(task)), p, pm);
-            ws_middle<RM, PLANE>(a + ws_pad(RM * p), a + ws_pad(RM * pm), t, a1, a2, be, task == 0,
-                                 H + 3 * WS_TASKS * RM);
+            ws_middle<RM, PLANE>(a + ws_pad(RM * p), a + ws_pad(RM * pm), t, h1, h2, task == 0, H + 2 * WS_TASKS * RM);
 #pragma unroll
             for (int s = 0; s < RM; ++s) {
-                a1[s] = n1[s];
-                a2[s] = n2[s];
-                be[s] = nb[s];
+                h1[s] = n1[s];
+                h2[s] = n2[s];
             }
             t = nt;
             task += 32;
