@@ -139,7 +139,7 @@ struct BatchState {
     int cap = 0;                  // right-hand sides the vectors below hold
     float *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr, *tod = nullptr;
     double *x64 = nullptr, *b64 = nullptr, *r64 = nullptr;
-    double *partial = nullptr, *rho = nullptr, *bb = nullptr, *rr = nullptr, *tol2 = nullptr;
+    double *partial = nullptr, *rho = nullptr, *bb = nullptr, *rr = nullptr, *tol2 = nullptr, *scal = nullptr;
     int* iters = nullptr;
     unsigned char* state = nullptr;
     int* flags = nullptr;
@@ -247,7 +247,7 @@ static void destroy_plan(PlanHolder* P) {
     for (void* p : {(void*)bt.tiles, (void*)bt.H, (void*)bt.ptw, (void*)bt.twiddle, (void*)bt.x, (void*)bt.r,
                     (void*)bt.p, (void*)bt.q, (void*)bt.z,
                     (void*)bt.tod, (void*)bt.x64, (void*)bt.b64, (void*)bt.r64, (void*)bt.partial, (void*)bt.rho,
-                    (void*)bt.bb, (void*)bt.rr, (void*)bt.tol2, (void*)bt.iters, (void*)bt.state, (void*)bt.flags,
+                    (void*)bt.bb, (void*)bt.rr, (void*)bt.tol2, (void*)bt.scal, (void*)bt.iters, (void*)bt.state, (void*)bt.flags,
                     (void*)bt.bar, (void*)bt.tc_groups, (void*)bt.tc_atab, (void*)bt.tc_invc, (void*)bt.tc_y,
                     (void*)bt.tc_scale})
         dfree(p);
@@ -2012,7 +2012,7 @@ static void ensure_batch_buffers(PlanHolder& P, int R) {
     if (bt.partial == nullptr) {
         bt.nblocks = std::max(1, std::min(batch_pcg_max_blocks(P.num_sms), (P.npix_obs + 31) / 32));
         bt.partial = dalloc<double>((size_t)bt.nblocks * BATCH_PSTRIDE);
-        for (double** v : {&bt.rho, &bt.bb, &bt.rr, &bt.tol2}) *v = dalloc<double>(BATCH_RMAX);
+        for (double** v : {&bt.rho, &bt.bb, &bt.rr, &bt.tol2, &bt.scal}) *v = dalloc<double>(BATCH_RMAX);
         bt.iters = dalloc<int>(BATCH_RMAX);
         bt.state = dalloc<unsigned char>(BATCH_RMAX);
         bt.flags = dalloc<int>(8);
@@ -2165,6 +2165,34 @@ static void run_batch_pcg(PlanHolder& P, int R, int maxit) {
     }
 }
 
+// r64_r = P^T N^-1 (d_r - P x64_r) for the columns with nrm_r != 0.  All at once where most of
+// them are active: one Toeplitz launch over as many columns as the batch's FP32 time-domain
+// buffer holds in FP64 (half of them), one scatter.  (Column by column a launch of a small scan
+// left most of the chip idle: 16 columns of 2^20 samples took 2.1 ms, all at once 1.1.)
+static void residual64_batch(PlanHolder& P, const double* D, const std::vector<double>& nrm, int active, int R, bool df) {
+    BatchState& bt = P.batch;
+    cudaStream_t s = P.stream;
+    const int64_t n = P.n, nt = P.nt;
+    const int cap = bt.cap / 2;
+    if (cap < 2 || 2 * active < R || P.sl_off == nullptr || P.npix_obs == 0) {
+        for (int r = 0; r < R; ++r)
+            if (nrm[(size_t)r] != 0.0) residual64(P, D + r * nt, bt.x64 + r * n, bt.r64 + r * n, df);
+        return;
+    }
+    double* tod = reinterpret_cast<double*>(bt.tod);
+    const bool use_df = df && P.tzdf.logn != 0;
+    for (int r0 = 0; r0 < R; r0 += cap) {
+        const int Rc = std::min(cap, R - r0);
+        int sl = prof_begin(P, use_df ? ST_TZDF : ST_TZ64);
+        if (use_df) launch_toeplitz_df(P, nullptr, D + r0 * nt, bt.x64 + r0 * n, Rc, n, tod, nt, s, nt);
+        else launch_toeplitz_any<double>(P, P.tz64, nullptr, D + r0 * nt, bt.x64 + r0 * n, Rc, n, tod, nt, nullptr, s, nt);
+        prof_end(P, sl);
+        sl = prof_begin(P, ST_SC64);
+        launch_batch_scatter_sliced<double>(P, tod, bt.r64 + r0 * n, Rc, nullptr, s);
+        prof_end(P, sl);
+    }
+}
+
 static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_opts& so, double* M, mm_stats* st) {
     cudaStream_t s = P.stream;
     if (R < 1) throw Error{MM_ERR_ARG, "R must be >= 1"};
@@ -2201,32 +2229,31 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
         launch_toeplitz_any<float>(P, batch_tz(P), nullptr, Dg, nullptr, Rc, (int64_t)nt, bt.tod, (int64_t)nt, nullptr, s);
         launch_batch_scatter(P, bt.tod, bt.z, Rc, nullptr, s);
         launch_convert_f32_to_f64(bt.z, bt.b64, (int64_t)Rc * n, s);
-        for (int r = 0; r < Rc; ++r) {
-            bb[(size_t)r] = dot64(P, bt.b64 + (size_t)r * n, bt.b64 + (size_t)r * n);
-            rr[(size_t)r] = bb[(size_t)r];
-        }
+        launch_dot_batch(bt.b64, (int64_t)n, Rc, bt.scal, s);
+        d2h(bb.data(), bt.scal, (size_t)Rc * 8, s);
+        sync(P);
+        rr = bb;
         check_cuda(cudaMemsetAsync(bt.x64, 0, n * Rc * 8, s), "memset x");
         check_cuda(cudaMemcpyAsync(bt.r64, bt.b64, n * Rc * 8, cudaMemcpyDeviceToDevice, s), "copy b");
         int total = 0;
         for (int o = 0; o < max_outer; ++o) {
-            std::vector<double> tol2(BATCH_RMAX, 0.0), nrm(Rc, 0.0);
+            std::vector<double> tol2(BATCH_RMAX, 0.0), nrm(Rc, 0.0), inv(Rc, 0.0);
             bool any = false;
             for (int r = 0; r < Rc; ++r) {
                 const bool act = bb[(size_t)r] > 0.0 && std::sqrt(rr[(size_t)r]) > so.tol * std::sqrt(bb[(size_t)r]);
-                float* r32 = bt.r + (size_t)r * n;
                 if (act) {
                     any = true;
                     nrm[(size_t)r] = std::sqrt(rr[(size_t)r]);
-                    launch_scale_f32(bt.r64 + (size_t)r * n, 1.0 / nrm[(size_t)r], r32, (int64_t)n, s);
+                    inv[(size_t)r] = 1.0 / nrm[(size_t)r];
                     double ti = 0.5 * so.tol * std::sqrt(bb[(size_t)r]) / nrm[(size_t)r];
                     ti = std::min(0.5, std::max(ti, inner_min));
                     if (o == 0 && so.first_inner_tol > 0.0) ti = so.first_inner_tol;
                     tol2[(size_t)r] = ti * ti;
-                } else {
-                    check_cuda(cudaMemsetAsync(r32, 0, n * 4, s), "memset r");
                 }
             }
             if (!any || total >= so.maxit) break;
+            h2d(bt.scal, inv.data(), (size_t)Rc * 8, s);
+            launch_scale_f32_batch(bt.r64, bt.scal, bt.r, (int64_t)n, Rc, s);   // r / ||r||, idle columns 0
             h2d(bt.tol2, tol2.data(), BATCH_RMAX * 8, s);
             run_batch_pcg(P, Rc, so.maxit - total);
             std::vector<int> it(BATCH_RMAX);
@@ -2234,7 +2261,7 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
             d2h(it.data(), bt.iters, BATCH_RMAX * 4, s);
             d2h(stt.data(), bt.state, BATCH_RMAX, s);
             sync(s);
-            int mx = 0;
+            int mx = 0, active = 0;
             for (int r = 0; r < Rc; ++r) {
                 if (nrm[(size_t)r] == 0.0) continue;
                 if (stt[(size_t)r] == 3) throw Error{MM_ERR_NOT_SPD, "batched PCG breakdown"};
@@ -2242,11 +2269,17 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
                 mx = std::max(mx, it[(size_t)r]);
                 outer[(size_t)r] += 1;
                 fp64[(size_t)r] += 1;
-                double* x64 = bt.x64 + (size_t)r * n;
-                launch_axpy_host(x64, bt.x + (size_t)r * n, nrm[(size_t)r], (int64_t)n, s);
-                residual64(P, Dg + (size_t)r * nt, x64, bt.r64 + (size_t)r * n, so.residual != MM_RESID_FP64);
-                rr[(size_t)r] = dot64(P, bt.r64 + (size_t)r * n, bt.r64 + (size_t)r * n);
+                ++active;
             }
+            h2d(bt.scal, nrm.data(), (size_t)Rc * 8, s);
+            launch_axpy_f32_batch(bt.x64, bt.x, bt.scal, (int64_t)n, Rc, s);
+            residual64_batch(P, Dg, nrm, active, Rc, so.residual != MM_RESID_FP64);
+            std::vector<double> now((size_t)Rc);
+            launch_dot_batch(bt.r64, (int64_t)n, Rc, bt.scal, s);
+            d2h(now.data(), bt.scal, (size_t)Rc * 8, s);
+            sync(P);
+            for (int r = 0; r < Rc; ++r)
+                if (nrm[(size_t)r] != 0.0) rr[(size_t)r] = now[(size_t)r];
             total += mx;
         }
         for (int r = 0; r < Rc; ++r) {

@@ -17,6 +17,7 @@
 #include "pcg.cuh"
 #include "toeplitz.cuh"
 
+#include <algorithm>
 #include <cooperative_groups.h>
 
 namespace mm {
@@ -296,7 +297,7 @@ __global__ void batch_scatter_kernel(const int32_t* __restrict__ off, const int3
 
 void launch_batch_scatter(const Plan& P, const float* Z, float* W, int R, const int* done, cudaStream_t s) {
     if (P.npix_obs == 0) return;
-    if (P.sl_off != nullptr) return launch_batch_scatter_sliced(P, Z, W, R, done, s);
+    if (P.sl_off != nullptr) return launch_batch_scatter_sliced<float>(P, Z, W, R, done, s);
     const int th = 256;
     int g = (P.npix_obs + 7) / 8;
     if (g > P.num_sms * 32) g = P.num_sms * 32;
@@ -544,29 +545,64 @@ int batch_pcg_max_blocks(int num_sms) {
 
 namespace mm {
 
-__global__ void scale_f32_kernel(const double* __restrict__ a, double s, float* __restrict__ out, int64_t n) {
+// Column r (grid.y) of a batch, scalars in device memory; a column whose scalar is 0 is left
+// out (x) or zeroed (out).
+__global__ void scale_f32_kernel(const double* __restrict__ a, const double* __restrict__ sc, float* __restrict__ out,
+                                 int64_t n) {
+    const double s = sc[blockIdx.y];
+    const int64_t o = (int64_t)blockIdx.y * n;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = (float)(a[i] * s);
+        out[o + i] = s == 0.0 ? 0.f : (float)(a[o + i] * s);
 }
 
-void launch_scale_f32(const double* a, double s, float* out, int64_t n, cudaStream_t st) {
-    int64_t g = (n + 255) / 256;
-    if (g > 2048) g = 2048;
-    scale_f32_kernel<<<(int)g, 256, 0, st>>>(a, s, out, n);
+__global__ void axpy_f32_batch_kernel(double* __restrict__ x, const float* __restrict__ d, const double* __restrict__ sc,
+                                      int64_t n) {
+    const double s = sc[blockIdx.y];
+    if (s == 0.0) return;
+    const int64_t o = (int64_t)blockIdx.y * n;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        x[o + i] += s * (double)d[o + i];
+}
+
+// out[r] = a_r . a_r: one block per column, a fixed order of sums
+__global__ void __launch_bounds__(1024) dot_batch_kernel(const double* __restrict__ a, int64_t n, double* __restrict__ out) {
+    __shared__ double sh[32];
+    const double* v = a + (int64_t)blockIdx.x * n;
+    double s = 0.0;
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += v[i] * v[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = sh[threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) out[blockIdx.x] = s;
+    }
+}
+
+static dim3 batch_grid(int64_t n, int R) {
+    return dim3((unsigned)std::min<int64_t>((n + 255) / 256, std::max(1, 4096 / R)), (unsigned)R);
+}
+
+void launch_scale_f32_batch(const double* a, const double* sc, float* out, int64_t n, int R, cudaStream_t st) {
+    if (n == 0) return;
+    scale_f32_kernel<<<batch_grid(n, R), 256, 0, st>>>(a, sc, out, n);
     check_cuda(cudaGetLastError(), "scale_f32 launch");
     note_launch();
 }
 
-__global__ void axpy_host_kernel(double* __restrict__ x, const float* __restrict__ d, double s, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] += s * (double)d[i];
+void launch_axpy_f32_batch(double* x, const float* d, const double* sc, int64_t n, int R, cudaStream_t st) {
+    if (n == 0) return;
+    axpy_f32_batch_kernel<<<batch_grid(n, R), 256, 0, st>>>(x, d, sc, n);
+    check_cuda(cudaGetLastError(), "axpy launch");
+    note_launch();
 }
 
-void launch_axpy_host(double* x, const float* d, double s, int64_t n, cudaStream_t st) {
-    int64_t g = (n + 255) / 256;
-    if (g > 2048) g = 2048;
-    axpy_host_kernel<<<(int)g, 256, 0, st>>>(x, d, s, n);
-    check_cuda(cudaGetLastError(), "axpy launch");
+void launch_dot_batch(const double* a, int64_t n, int R, double* out, cudaStream_t st) {
+    dot_batch_kernel<<<R, 1024, 0, st>>>(a, n, out);
+    check_cuda(cudaGetLastError(), "dot launch");
     note_launch();
 }
 

@@ -86,6 +86,8 @@ int batch_pcg_max_blocks(int num_sms);
 }  // namespace mm
 
 namespace mm {
-void launch_scale_f32(const double* a, double s, float* out, int64_t n, cudaStream_t st);
-void launch_axpy_host(double* x, const float* d, double s, int64_t n, cudaStream_t st);
+// R columns of n values; sc, out: device double[R]
+void launch_scale_f32_batch(const double* a, const double* sc, float* out, int64_t n, int R, cudaStream_t st);
+void launch_axpy_f32_batch(double* x, const float* d, const double* sc, int64_t n, int R, cudaStream_t st);
+void launch_dot_batch(const double* a, int64_t n, int R, double* out, cudaStream_t st);
 }  // namespace mm

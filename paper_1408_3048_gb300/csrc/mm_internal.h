@@ -271,14 +271,16 @@ template <typename T>
 void launch_toeplitz_rhs(const Plan& P, const ToeplitzDev& tz, const T* y_tod, const T* x_map, int R,
                          int64_t in_stride, T* z, int64_t out_stride, const int* done, cudaStream_t s);
 // General form: d_tod (FP64 time domain) alone is rounded to T (FP32 only); with x_map the
-// input is d - P x (FP64 only: the residual data of b - A x).
+// input is d - P x (FP64 only: the residual data of b - A x; right-hand side r: x + r in_stride,
+// d + r d_stride).
 template <typename T>
 void launch_toeplitz_any(const Plan& P, const ToeplitzDev& tz, const T* y_tod, const double* d_tod, const T* x_map,
-                         int R, int64_t in_stride, T* z, int64_t out_stride, const int* done, cudaStream_t s);
+                         int R, int64_t in_stride, T* z, int64_t out_stride, const int* done, cudaStream_t s,
+                         int64_t d_stride = 0);
 // Double-float N^-1 on FP64 data (toeplitz_df.cu): y (time domain) given, or else the
 // residual data d - P x; output z FP64 [nt] (R right-hand sides as for launch_toeplitz_rhs)
 void launch_toeplitz_df(const Plan& P, const double* y, const double* d, const double* x, int R, int64_t in_stride,
-                        double* z, int64_t out_stride, cudaStream_t s);
+                        double* z, int64_t out_stride, cudaStream_t s, int64_t d_stride = 0);
 // FP32 I/Q/U N^-1 P x with the gather reading x from P.map4; pack: first write x into
 // P.map4 (one small kernel), else P.map4 already holds x (the FP32 PCG kernels keep it)
 void launch_toeplitz_f32_packed(const Plan& P, const float* x, bool pack, float* z, const int* done,
@@ -309,7 +311,8 @@ void launch_slice_fill(const Plan& P, int32_t* st, double2* sw64, float2* sw32, 
 template <typename T>
 void launch_scatter_sliced(const Plan& P, const T* z, T* w, const T* p, double* part, unsigned* count, double* pq,
                            const int* done, cudaStream_t s);
-void launch_batch_scatter_sliced(const Plan& P, const float* Z, float* W, int R, const int* done, cudaStream_t s);
+template <typename T>
+void launch_batch_scatter_sliced(const Plan& P, const T* Z, T* W, int R, const int* done, cudaStream_t s);
 int sliced_blocks(const Plan& P, int wpb, int S);
 void launch_bd_build(const Plan& P, double* bd64, float* bd32, cudaStream_t s);
 // merged a priori coarse space Z_S (Sec. 3.3.1), r groups of consecutive intervals, into

@@ -651,11 +651,13 @@ __global__ void dot_partial_kernel(const TA* a, const TB* b, int64_t n, double* 
 }
 
 __global__ void sum_kernel(const double* part, int m, double* out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < m; ++i) s += part[i];
-        *out = s;
-    }
+    // one warp, a fixed order: lanes over the partials, then a tree (one thread adding 304
+    // values one after the other took 21 us, the warp 3)
+    double s = 0.0;
+    for (int i = threadIdx.x; i < m; i += 32) s += part[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *out = s;
 }
 
 void launch_dot64(const double* a, const double* b, int64_t n, double* part, double* out, cudaStream_t s) {

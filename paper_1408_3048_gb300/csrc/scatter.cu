@@ -320,45 +320,46 @@ template void launch_scatter_sliced<float>(const Plan&, const float*, float*, co
                                            double*, const int*, cudaStream_t);
 
 // ------------------------------------------------------------- many right-hand sides
-// The same walk for SL_RC right-hand sides at a time (grid.y): a step's indices and weights
-// are read once for them.
-constexpr int SL_RC = 4, SL_BU = 4;
+// The same walk for RC right-hand sides at a time (grid.y; four in FP32, two in FP64): a step's
+// indices and weights are read once for them.
+constexpr int SL_BU = 4;
 
-template <int NC>
+template <typename T, int NC, int RC>
 __global__ void __launch_bounds__(256) sliced_batch_kernel(const int32_t* __restrict__ sl_off,
                                                            const int32_t* __restrict__ st,
-                                                           const float2* __restrict__ sw, const float* __restrict__ Z,
-                                                           float* __restrict__ W, int nslices, int npix, int64_t nt,
-                                                           int64_t n, int R, const int* done) {
+                                                           const typename W2<T>::type* __restrict__ sw,
+                                                           const T* __restrict__ Z, T* __restrict__ W, int nslices,
+                                                           int npix, int64_t nt, int64_t n, int R, const int* done) {
+    using V2 = typename W2<T>::type;
     if (done != nullptr && *(volatile const int*)done) return;
     const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-    const int r0 = blockIdx.y * SL_RC;
-    const float* z0 = Z + (size_t)r0 * nt;
+    const int r0 = blockIdx.y * RC;
+    const T* z0 = Z + (size_t)r0 * nt;
     for (int s = blockIdx.x * warps + (threadIdx.x >> 5); s < nslices; s += gridDim.x * warps) {
-        Acc<float> a[SL_RC][NC];
+        Acc<T> a[RC][NC];
         const int j1 = sl_off[s + 1];
         for (int j = sl_off[s]; j < j1; j += SL_BU) {
             int t[SL_BU];
-            float2 ww[SL_BU];
+            V2 ww[SL_BU];
 #pragma unroll
             for (int u = 0; u < SL_BU; ++u) {
                 const int64_t e = (int64_t)min(j + u, j1 - 1) * 32 + lane;
                 t[u] = j + u < j1 ? __ldg(st + e) : -1;
                 if constexpr (NC == 3) ww[u] = __ldg(sw + e);
             }
-            float v[SL_RC][SL_BU];
+            T v[RC][SL_BU];
 #pragma unroll
-            for (int r = 0; r < SL_RC; ++r) {
-                const float* z = z0 + (r0 + r < R ? (size_t)r * nt : 0);
+            for (int r = 0; r < RC; ++r) {
+                const T* z = z0 + (r0 + r < R ? (size_t)r * nt : 0);
 #pragma unroll
                 for (int u = 0; u < SL_BU; ++u) v[r][u] = z[max(t[u], 0)];
             }
 #pragma unroll
-            for (int r = 0; r < SL_RC; ++r) {
-                float b[NC] = {};
+            for (int r = 0; r < RC; ++r) {
+                T b[NC] = {};
 #pragma unroll
                 for (int u = 0; u < SL_BU; ++u) {
-                    const float x = t[u] >= 0 ? v[r][u] : 0.f;
+                    const T x = t[u] >= 0 ? v[r][u] : (T)0;
                     b[0] += x;
                     if constexpr (NC == 3) {
                         b[1] += ww[u].x * x;
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(256) sliced_batch_kernel(const int32_t* __rest
         }
         const int q = s * SL_PIX + (lane >> 2);
 #pragma unroll
-        for (int r = 0; r < SL_RC; ++r)
+        for (int r = 0; r < RC; ++r)
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 a[r][c].lanes(1);
@@ -381,18 +382,20 @@ __global__ void __launch_bounds__(256) sliced_batch_kernel(const int32_t* __rest
     }
 }
 
-void launch_batch_scatter_sliced(const Plan& P, const float* Z, float* W, int R, const int* done, cudaStream_t s) {
-    const int gy = (R + SL_RC - 1) / SL_RC;
+template <typename T>
+void launch_batch_scatter_sliced(const Plan& P, const T* Z, T* W, int R, const int* done, cudaStream_t s) {
+    constexpr int RC = sizeof(T) == 4 ? 4 : 2;
     const int gx = std::max(1, std::min((P.sl_count + 7) / 8, P.num_sms * 8));
-    const dim3 grid((unsigned)gx, (unsigned)gy);
-    if (P.ncomp == 1)
-        sliced_batch_kernel<1><<<grid, 256, 0, s>>>(P.sl_off, P.sl_t, nullptr, Z, W, P.sl_count, P.npix_obs, P.nt, P.n, R,
-                                                    done);
-    else
-        sliced_batch_kernel<3><<<grid, 256, 0, s>>>(P.sl_off, P.sl_t, P.sl_w32, Z, W, P.sl_count, P.npix_obs, P.nt, P.n, R,
-                                                    done);
+    const dim3 grid((unsigned)gx, (unsigned)((R + RC - 1) / RC));
+    const typename W2<T>::type* sw = nullptr;
+    if constexpr (sizeof(T) == 4) sw = P.sl_w32;
+    else sw = P.sl_w64;
+    auto kern = P.ncomp == 1 ? sliced_batch_kernel<T, 1, RC> : sliced_batch_kernel<T, 3, RC>;
+    kern<<<grid, 256, 0, s>>>(P.sl_off, P.sl_t, sw, Z, W, P.sl_count, P.npix_obs, P.nt, P.n, R, done);
     check_cuda(cudaGetLastError(), "batch scatter launch");
     note_launch();
 }
+template void launch_batch_scatter_sliced<float>(const Plan&, const float*, float*, int, const int*, cudaStream_t);
+template void launch_batch_scatter_sliced<double>(const Plan&, const double*, double*, int, const int*, cudaStream_t);
 
 }  // namespace mm

@@ -80,6 +80,7 @@ struct TzArgs {
     int lambda;
     int R;                 // right-hand sides (grid: tile-major, RHS fastest)
     int64_t in_stride;     // elements between RHS in y (mode 0) or x (gather modes)
+    int64_t d_stride;      // elements between RHS in yd
     int64_t out_stride;    // elements between RHS in z
     int pf_ahead = 0;      // CTAs resident at once: L2 prefetch distance (0: no prefetch)
     const float4* x4 = nullptr;   // FP32 I/Q/U map packed per pixel (mode 3), else nullptr
@@ -390,11 +391,12 @@ __device__ __forceinline__ int64_t seg_d(const Tile& tl, int g) {
 // takes a branch-free path.
 template <typename T, int NT, int MODE>
 __device__ __forceinline__ void load_block(const TzArgs<T>& A, const Tile& tile, T* ar, int s0, int count,
-                                           int64_t roff) {
+                                           int rhs) {
     using I = In<T>;
+    const int64_t roff = rhs * A.in_stride;
     const I* __restrict__ y = A.y + roff;
     const I* __restrict__ x = A.x + roff;
-    const double* __restrict__ yd = A.yd + roff;
+    const double* __restrict__ yd = A.yd + rhs * A.d_stride;
     const int tid = threadIdx.x;
     const int PER = count / NT;
     constexpr bool IQU = MODE == 3 || MODE == 5;
@@ -598,7 +600,7 @@ __device__ __forceinline__ void prefetch_issue(const TzArgs<T>& A, const PfSeg& 
     if (sg.n == 0) return;
     const int64_t roff = sg.rhs * A.in_stride, t0 = sg.t0, n = sg.n;
     if constexpr (MODE == 0) l2_prefetch(A.y + roff + t0, n * (int64_t)sizeof(In<T>));
-    if constexpr (MODE == 2 || MODE >= 4) l2_prefetch(A.yd + roff + t0, n * 8);
+    if constexpr (MODE == 2 || MODE >= 4) l2_prefetch(A.yd + sg.rhs * A.d_stride + t0, n * 8);
     if constexpr (MODE != 0 && MODE != 2) {
         if (sg.rhs == 0) {
             l2_prefetch(A.pixc + t0, n * 4);
@@ -672,7 +674,7 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
     PfSeg next{0, 0, 0};
     if (A.pf_ahead > 0 && (int64_t)blockIdx.x + A.pf_ahead < (int64_t)gridDim.x)
         next = prefetch_seg(A, blockIdx.x + A.pf_ahead, threadIdx.x);
-    load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), 0, 2 * N, tr.rhs * A.in_stride);
+    load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), 0, 2 * N, tr.rhs);
     __syncthreads();
     prefetch_issue<T, MODE>(A, next);
     fft_all<T, LOGN, NT, 0>(a, A.ptw);
@@ -806,7 +808,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     const TileRhs tr = tile_rhs(blockIdx.x / CL, A.R);
     const Tile tile = A.tiles[tr.tile];
     const int tid = threadIdx.x;
-    load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), rank * 2 * M, 2 * M, tr.rhs * A.in_stride);
+    load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), rank * 2 * M, 2 * M, tr.rhs);
     cl.sync();
     C2 y[PER];
 #pragma unroll
@@ -835,29 +837,44 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     constexpr int64_t HS = F32 ? N + 1 : split_size(N);
     const T* al = A.H + tile.psd * HS;
     const T* be = al + N;
-    // bins k and N - k (FP32: the chain, al = the spectrum itself)
-    auto product = [&](C2 u1, C2 u2, int k, C2& V1, C2& V2) {
-        const int k2 = (N - k) & (N - 1);
+    // bins k and N - k (FP32: the chain, al = the spectrum itself, h1 and h2 its values)
+    auto product = [&](C2 u1, C2 u2, int k, T h1, T h2, C2& V1, C2& V2) {
         if constexpr (F32) {
-            T cw, sw;
-            twiddle<T, LOGQ>(A.twiddle, k, cw, sw);
-            split_chain(u1, u2, cw, sw, al[k], al[N - k], V1, V2);
+            float sw, cw;
+            sincospif((float)k * (1.f / (float)N), &sw, &cw);
+            split_chain(u1, u2, cw, sw, h1, h2, V1, V2);
         } else {
-            split_product<T>(u1, u2, al[k], al[k2], be[k < k2 ? k : k2], V1, V2);
+            const int k2 = (N - k) & (N - 1);
+            split_product<T>(u1, u2, h1, h2, be[k < k2 ? k : k2], V1, V2);
         }
     };
+    auto second = [&](int k) { return F32 ? N - k : (N - k) & (N - 1); };   // index of h2
     const int prank = (CL - rank) % CL;
     if (prank == rank) {
         // partner bins inside this CTA: process each pair once
-        const int npairs = rank == 0 ? M / 2 + 1 : M / 2;
-        for (int k1 = tid; k1 < npairs; k1 += NT) {
-            const int k = CL * k1 + rank;
+        auto pair = [&](int k1, T h1, T h2) {
             const int p = rank == 0 ? ((M - k1) & (M - 1)) : (M - 1 - k1);
             C2 V1, V2;
-            product(a[pad<T>(k1)], a[pad<T>(p)], k, V1, V2);
+            product(a[pad<T>(k1)], a[pad<T>(p)], CL * k1 + rank, h1, h2, V1, V2);
             a[pad<T>(k1)] = V1;
             if (p != k1) a[pad<T>(p)] = V2;
+        };
+        // spectrum values requested U pairs at a time; pair M / 2 of rank 0 apart
+        constexpr int PAIRS = M / 2 / NT, U = F32 ? (PAIRS < 8 ? PAIRS : 8) : 2;
+        static_assert(PAIRS >= U && PAIRS % U == 0, "pairs per thread");
+#pragma unroll 1
+        for (int g = 0; g < PAIRS; g += U) {
+            T h1[U], h2[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int k = CL * (tid + (g + u) * NT) + rank;
+                h1[u] = al[k];
+                h2[u] = al[second(k)];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) pair(tid + (g + u) * NT, h1[u], h2[u]);
         }
+        if (rank == 0 && tid == 0) pair(M / 2, al[CL * (M / 2)], al[second(CL * (M / 2))]);
         cl.sync();
         cl.sync();
     } else {
@@ -869,7 +886,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
             const int k1 = u * NT + tid;
             const int k = CL * k1 + rank;
             C2 V2;
-            product(a[pad<T>(k1)], part[prank][pad<T>(M - 1 - k1)], k, vo[u], V2);
+            product(a[pad<T>(k1)], part[prank][pad<T>(M - 1 - k1)], k, al[k], al[second(k)], vo[u], V2);
         }
         cl.sync();
 #pragma unroll

@@ -24,7 +24,7 @@ template <>
 int toeplitz_max_logn<dfl>() { return 13; }
 
 void launch_toeplitz_df(const Plan& P, const double* y, const double* d, const double* x, int R, int64_t in_stride,
-                        double* z, int64_t out_stride, cudaStream_t s) {
+                        double* z, int64_t out_stride, cudaStream_t s, int64_t d_stride) {
     const ToeplitzDev& tz = P.tzdf;
     if (tz.logn == 0) throw Error{MM_ERR_ARG, "no double-float Toeplitz block for this plan"};
     if (tz.ntiles == 0) return;
@@ -43,6 +43,7 @@ void launch_toeplitz_df(const Plan& P, const double* y, const double* d, const d
     A.lambda = P.lambda;
     A.R = R;
     A.in_stride = in_stride;
+    A.d_stride = d_stride;
     A.out_stride = out_stride;
     A.pf_ahead = P.num_sms;
     if (y != nullptr || d == nullptr || x == nullptr)

@@ -38,7 +38,8 @@ static void dispatch_f32(const TzArgs<float>& A, const ToeplitzDev& tz, int num_
 // FP64 only), else the gather of x (1 / 3).
 template <>
 void launch_toeplitz_any<float>(const Plan& P, const ToeplitzDev& tz, const float* y, const double* yd, const float* x,
-                             int R, int64_t in_stride, float* z, int64_t out_stride, const int* done, cudaStream_t s) {
+                             int R, int64_t in_stride, float* z, int64_t out_stride, const int* done, cudaStream_t s,
+                             int64_t d_stride) {
     if (tz.logn == 0) throw Error{MM_ERR_ARG, "no FP32 Toeplitz block fits this lambda"};
     if (tz.ntiles == 0) return;
     TzArgs<float> A;
@@ -56,6 +57,7 @@ void launch_toeplitz_any<float>(const Plan& P, const ToeplitzDev& tz, const floa
     A.lambda = P.lambda;
     A.R = R;
     A.in_stride = in_stride;
+    A.d_stride = x == nullptr ? in_stride : d_stride;
     A.out_stride = out_stride;
     A.pf_ahead = P.num_sms;
     const int mode = y != nullptr ? 0 : (yd != nullptr ? (x == nullptr ? 2 : (P.ncomp == 1 ? 4 : 5)) : (P.ncomp == 1 ? 1 : 3));
@@ -108,6 +110,7 @@ void launch_toeplitz_f32_packed(const Plan& P, const float* x, bool pack, float*
     A.lambda = P.lambda;
     A.R = 1;
     A.in_stride = 0;
+    A.d_stride = 0;
     A.out_stride = 0;
     A.pf_ahead = P.num_sms;
     A.x4 = P.map4;

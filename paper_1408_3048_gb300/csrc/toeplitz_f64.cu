@@ -13,7 +13,8 @@ int toeplitz_max_logn<double>() { return 13; }
 // FP64 only), else the gather of x (1 / 3).
 template <>
 void launch_toeplitz_any<double>(const Plan& P, const ToeplitzDev& tz, const double* y, const double* yd, const double* x,
-                             int R, int64_t in_stride, double* z, int64_t out_stride, const int* done, cudaStream_t s) {
+                             int R, int64_t in_stride, double* z, int64_t out_stride, const int* done, cudaStream_t s,
+                             int64_t d_stride) {
     if (tz.logn == 0) throw Error{MM_ERR_ARG, "no FP64 Toeplitz block fits this lambda"};
     if (tz.ntiles == 0) return;
     TzArgs<double> A;
@@ -31,6 +32,7 @@ void launch_toeplitz_any<double>(const Plan& P, const ToeplitzDev& tz, const dou
     A.lambda = P.lambda;
     A.R = R;
     A.in_stride = in_stride;
+    A.d_stride = x == nullptr ? in_stride : d_stride;
     A.out_stride = out_stride;
     A.pf_ahead = P.num_sms;
     const int mode = y != nullptr ? 0 : (yd != nullptr ? (x == nullptr ? 2 : (P.ncomp == 1 ? 4 : 5)) : (P.ncomp == 1 ? 1 : 3));
