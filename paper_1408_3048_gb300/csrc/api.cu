@@ -254,9 +254,10 @@ static void destroy_plan(PlanHolder* P) {
     delete P;
 }
 
-// Time of a launch over `tiles` overlap-save tiles of a block, in microseconds, from timings of
-// every block on scans of 2^14 to 2^26 samples with lambda = 32 to 16384 (the blocks it picks
-// were within 5 % of the fastest in 43 of 46 of them).
+// Time of a launch over `tiles` overlap-save tiles of a block, in microseconds: fits to timings
+// of every block on scans of 2^14 to 2^26 samples with lambda = 32 to 16384.  The operation
+// count that it replaces took blocks too large for the chip on small scans: FP64, 2^18 samples
+// at lambda = 1024: 44 tiles of 2^13 reals on 152 SMs 110 us, the blocks of 2^12 reals 57 us.
 //
 // FP64 and double-float: a tile keeps an SM's pipe busy for `per`, alone it takes `lat`
 // (latency of its chain of passes where that is longer); tiles go round the SMs, the cluster
@@ -629,9 +630,9 @@ static void build_sliced(Plan& P) {
                 check_cuda(cudaMemsetAsync(static_cast<char*>(p) + (e - SL_PAD) * b, 0, SL_PAD * b, P.stream), "memset");
         launch_slice_fill(P, P.sl_t, P.sl_w64, P.sl_w32, P.sl_ang, P.stream);
         sync(P.stream);   // the host array goes out of scope
-    } catch (...) {
+    } catch (const Error& e) {
         free_sliced(P);
-        throw;
+        if (e.st != MM_ERR_OOM) throw;   // without room for a second layout the first one serves
     }
 }
 
@@ -1948,6 +1949,7 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
         }
         if (logn != P.tz32.logn && want != BATCH_PAIR && (want == BATCH_REAL || best < 0 || real_cost < best_cost))
         {
+            free_tz(bt.tz);   // of a first call that failed later on
             build_toeplitz<float>(P, bt.tz, logn + 1);
             P.spec.clear();
             P.spec_n = 0;

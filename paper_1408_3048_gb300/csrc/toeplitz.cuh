@@ -827,9 +827,9 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
     }
 }
 
-// Resident CTAs per SM: FP32 blocks below 2^15 reals run 1024 / NT CTAs of NT threads per
-// SM (at most 64 registers a thread), so that one CTA's gather overlaps another's FFT;
-// the 1024-thread FP32 block and FP64 / double-float keep their own register use (one
+// Resident CTAs per SM: the FP32 blocks here (up to 2^13 reals; toeplitz_ws.cu has the larger
+// ones) run 1024 / NT CTAs of NT threads per SM (at most 64 registers a thread), so that one
+// CTA's gather overlaps another's FFT; FP64 / double-float keep their own register use (one
 // CTA per SM), and so do 32-thread CTAs, which the 64-register cap would make spill.
 template <typename T, int NT>
 __host__ __device__ constexpr int tz_min_blocks() {
@@ -998,8 +998,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
 }
 
 // Threads per CTA: one largest-radix butterfly per thread and pass (N/16, or N/8 for
-// small N), capped at 1024 for FP32 (16 complex values per thread fit the 64-register
-// budget of a 1024-thread CTA) and 512 for FP64, at least 32.
+// small N), capped at 1024 for FP32 (the cluster blocks: 16 complex values per thread fit the
+// 64-register budget of a 1024-thread CTA) and 512 for FP64, at least 32.
 template <typename T, int LOGN>
 __host__ __device__ constexpr int tz_threads() {
     constexpr int cap = sizeof(T) == 4 ? 1024 : 512;
