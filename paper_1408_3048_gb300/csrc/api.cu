@@ -1958,7 +1958,10 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
     if (best < 0 && real_cost < 0.0) throw Error{MM_ERR_ARG, "lambda too large for the batched FFT blocks"};
     if ((want == BATCH_PAIR && best < 0) || (want == BATCH_REAL && real_cost < 0.0))
         throw Error{MM_ERR_ARG, "no FFT block supports this batched form for lambda"};
-    if (best >= 0) build_batch_pair(P, best);
+    // the pair form's tables where it is asked for, timed or the cheaper one (a first batched call
+    // of 64 columns on 2^22 samples otherwise spends 1.8 ms on tables that nothing reads)
+    if (want >= 0 ? want == BATCH_PAIR : best >= 0 && (P.autotune || real_cost < 0.0 || best_cost <= real_cost))
+        build_batch_pair(P, best);
     if (want >= 0) {
         bt.kind = want;
     } else if (best < 0) {
