@@ -189,11 +189,11 @@ def fft_tiles(scan, B, max_segments=3):
 # Sources whose text fixes each profiled kernel: the DRAM traffic recorded from an ncu capture
 # (a "traffic:" line in profiles/*.md) is reported only while their hash is unchanged.
 KERNEL_SOURCES = {
-    "toeplitz_f32": ["toeplitz.cuh", "toeplitz_f32.cu"],
+    "toeplitz_f32": ["toeplitz.cuh", "toeplitz_f32.cu", "toeplitz_ws.cu"],
     "toeplitz_f64": ["toeplitz.cuh", "toeplitz_f64.cu"],
     "toeplitz_df": ["toeplitz.cuh", "dfloat.cuh", "toeplitz_df.cu", "toeplitz_df_cluster.cu"],
-    "scatter_f32": ["pointing.cu"],
-    "scatter_f64": ["pointing.cu"],
+    "scatter_f32": ["pointing.cu", "scatter.cu"],
+    "scatter_f64": ["pointing.cu", "scatter.cu"],
     "pcg_f32": ["pcg.cu", "pcg.cuh"],
     "pcg_f64": ["pcg.cu", "pcg.cuh"],
 }
