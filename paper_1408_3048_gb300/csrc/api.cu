@@ -2014,16 +2014,19 @@ static void ensure_batch_buffers(PlanHolder& P, int R) {
     for (float** v : {&bt.x, &bt.r, &bt.p, &bt.q, &bt.z}) *v = dalloc<float>(n * R);
     bt.tod = dalloc<float>(nt * R);
     for (double** v : {&bt.x64, &bt.b64, &bt.r64}) *v = dalloc<double>(n * R);
-    if (bt.partial == nullptr) {
-        bt.nblocks = std::max(1, std::min(batch_pcg_max_blocks(P.num_sms), (P.npix_obs + 31) / 32));
-        bt.partial = dalloc<double>((size_t)bt.nblocks * BATCH_PSTRIDE);
-        for (double** v : {&bt.rho, &bt.bb, &bt.rr, &bt.tol2, &bt.scal}) *v = dalloc<double>(BATCH_RMAX);
-        bt.iters = dalloc<int>(BATCH_RMAX);
-        bt.state = dalloc<unsigned char>(BATCH_RMAX);
-        bt.flags = dalloc<int>(8);
-        bt.bar = dalloc<unsigned>(4);
-        check_cuda(cudaMemsetAsync(bt.bar, 0, 16, P.stream), "memset");
-    }
+    // the small buffers each on its own: a call that ran out of memory between two of them is
+    // followed by one that allocates the rest
+    bt.nblocks = std::max(1, std::min(batch_pcg_max_blocks(P.num_sms), (P.npix_obs + 31) / 32));
+    auto once = [](auto*& v, size_t count) {
+        if (v == nullptr) v = static_cast<std::remove_reference_t<decltype(v)>>(dmalloc(count * sizeof(*v)));
+    };
+    once(bt.partial, (size_t)bt.nblocks * BATCH_PSTRIDE);
+    for (double** v : {&bt.rho, &bt.bb, &bt.rr, &bt.tol2, &bt.scal}) once(*v, BATCH_RMAX);
+    once(bt.iters, BATCH_RMAX);
+    once(bt.state, BATCH_RMAX);
+    once(bt.flags, 8);
+    once(bt.bar, 4);
+    check_cuda(cudaMemsetAsync(bt.bar, 0, 16, P.stream), "memset");
     bt.cap = R;
 }
 

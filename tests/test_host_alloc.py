@@ -1,0 +1,121 @@
+"""Allocation failures in the library's host code, on the CPU: the library's objects linked with
+a CUDA runtime of host memory and kernels that do nothing (fake_cuda.cpp).  Every allocation
+of a call is made to fail in turn; the call reports MM_ERR_OOM (or does without), what it
+held is given back, and the next calls launch with live tables only."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1408_3048_gb300 import build, mm
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    inc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    if shutil.which("g++") is None or not os.path.isdir(inc):
+        pytest.skip("g++ or the CUDA headers not available")
+    build.build()
+    objs = [os.path.join(build.BUILD, f) for f in sorted(os.listdir(build.BUILD)) if f.endswith(".o")]
+    so = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-I", inc, "-o", so,
+                    os.path.join(HERE, "fake_cuda.cpp"), *objs, "-lpthread"], check=True)
+    L = ctypes.CDLL(so)
+    for name, (res, args) in mm._SIGS.items():
+        fn = getattr(L, name)
+        fn.restype, fn.argtypes = res, args
+    for name in ("fake_live_bytes", "fake_peak_bytes"):
+        getattr(L, name).restype = ctypes.c_longlong
+    L.fake_fail_after.argtypes = [ctypes.c_longlong]
+    L.fake_launch_name.restype = ctypes.c_char_p
+    return L
+
+
+class Plan:
+    """A plan of the fake device: two detectors of `lengths` each."""
+
+    def __init__(self, L, lengths, lam, ncomp=3, side=16, npsd=2, psd_of=None, expect=mm.MM_OK, **opts):
+        self.L = L
+        lengths = list(lengths) * 2
+        self.nt = sum(lengths)
+        pix = (np.arange(self.nt) // 4 % (side * side)).astype(np.int32)
+        phi = np.arange(self.nt) * 0.618
+        w = np.stack([np.cos(2 * phi), np.sin(2 * phi)], 1) if ncomp == 3 else None
+        off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+        ipsd = (np.arange(len(lengths)) * npsd // len(lengths)).astype(np.int32)
+        psd = (mm.mm_psd * npsd)(*[mm.mm_psd(1.0, 0.5, 1.0)] * npsd)
+        o = mm.mm_opts(ncomp=ncomp, lambda_=lam, fsamp=100.0, **opts)
+        self.h = ctypes.c_void_p()
+        self.status = L.mm_plan(ctypes.byref(self.h), pix.ctypes.data, self.nt, side * side,
+                                None if w is None else w.ctypes.data, off.ctypes.data, off.size - 1, ipsd.ctypes.data, psd,
+                                npsd, ctypes.byref(o))
+        assert self.status == expect
+        if self.status == mm.MM_OK:
+            n = ctypes.c_int64()
+            b64, b32 = ctypes.c_int32(), ctypes.c_int32()
+            L.mm_plan_info(self.h, None, ctypes.byref(n), None, ctypes.byref(b64), ctypes.byref(b32))
+            self.n, self.block64, self.block32 = n.value, b64.value, b32.value
+            self.X = np.zeros(64 * self.n, dtype=np.float32)
+
+    def batch(self, R):
+        """Status of Y = A X on R columns, and the launches of it."""
+        self.L.fake_clear_launches()
+        st = self.L.mm_apply_A_batch(self.h, R, self.X.ctypes.data, self.X.ctypes.data)
+        return st, launches(self.L)
+
+    def solve_batch(self, R):
+        self.L.fake_clear_launches()
+        D, M = np.zeros((R, self.nt)), np.zeros((R, self.n))
+        o = mm.mm_solve_opts(tol=1e-6, maxit=10, kind=mm.MM_PREC_BD, solver=mm.MM_SOLVE_MIXED)
+        st = self.L.mm_solve_batch(self.h, D.ctypes.data, R, ctypes.byref(o), M.ctypes.data, None)
+        return st, launches(self.L)
+
+    def config(self, R, kind=-1):
+        """(form, log2 block) of the batched operator."""
+        k, b = ctypes.c_int32(kind), ctypes.c_int32()
+        st = self.L.mm_batch_config(self.h, R, ctypes.byref(k), ctypes.byref(b), None)
+        assert st == mm.MM_OK
+        return k.value, b.value
+
+    def close(self):
+        self.L.mm_destroy(self.h)
+
+
+def launches(L):
+    return [(L.fake_launch_name(i).decode(), L.fake_launch_grid(i), L.fake_launch_dead(i)) for i in range(L.fake_launches())]
+
+
+def dead(ls):
+    return [l for l in ls if l[2] != 0]
+
+
+# (interval lengths, lambda, components): at 64 columns the pair form
+BATCHES = [([9000, 9000], 500, 3)]
+
+
+@pytest.mark.parametrize("lengths,lam,ncomp", BATCHES)
+def test_batched_call_without_memory(lib, lengths, lam, ncomp):
+    """A first batched call with each of its allocations failing in turn: it fails or does without,
+    and later calls, on fewer columns too (which take other tables), launch with live ones."""
+    base, failed = lib.fake_live_bytes(), 0
+    for k in range(60):
+        p = Plan(lib, lengths, lam, ncomp)
+        lib.fake_fail_after(k)
+        st, ls = p.batch(64)
+        done = lib.fake_fail_after(-1) != 0
+        assert st in (mm.MM_OK, mm.MM_ERR_OOM) and not dead(ls), k
+        failed += st == mm.MM_ERR_OOM
+        for call in (p.batch, p.solve_batch):
+            for R in (1, 2, 64):
+                st, ls = call(R)
+                assert st == mm.MM_OK and not dead(ls), (k, R, dead(ls))
+        p.close()
+        assert lib.fake_live_bytes() == base, k
+        if done:
+            break
+    assert failed >= 17 and done
