@@ -1896,6 +1896,30 @@ static void ensure_batch_tc_buffer(PlanHolder& P, int R) {
 static void launch_batch_tz(PlanHolder& P, int R, const float* X, float* Z, const int* done);
 static const ToeplitzDev& batch_tz(const PlanHolder& P) { return P.batch.tz.logn != 0 ? P.batch.tz : P.tz32; }
 
+// The real form's own block, complete or (false) not at all: without memory for it the plan's
+// block serves.
+static bool build_batch_real(PlanHolder& P, int logn) {
+    ToeplitzDev t;
+    bool ok = false;
+    try {
+        build_toeplitz<float>(P, t, logn + 1);
+        ok = true;
+    } catch (const Error& e) {
+        if (e.st != MM_ERR_OOM) {
+            free_tz(t);
+            throw;
+        }
+    } catch (...) {
+        free_tz(t);
+        throw;
+    }
+    P.spec.clear();
+    P.spec_n = 0;
+    if (!ok) free_tz(t);
+    else P.batch.tz = t;
+    return ok;
+}
+
 // Batched Toeplitz form, chosen once per plan (before any graph capture), after the
 // R-column buffers exist:
 //   BATCH_PAIR  two RHS per complex FFT (y_a + i y_b, one complex block of 2^logb points,
@@ -1936,10 +1960,12 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
     }
     // the real form's block for this many right-hand sides: one that fills the chip with R
     // launches' worth of tiles can be larger than the one with the shortest single launch
+    free_tz(bt.tz);   // of a first call that failed later on
     double real_cost = -1.0;
     if (P.tz32.logn != 0) {
+        const double own_cost = block_us<float>(P, P.tz32.logn, (int64_t)P.tz32.ntiles * R);
         int logn = P.tz32.logn;
-        real_cost = block_us<float>(P, logn, (int64_t)P.tz32.ntiles * R);
+        real_cost = own_cost;
         if (!P.forced_f32 && !P.autotune) {
             const auto c = block_candidates<float>(P, R);
             if (c[0].first < 0.95 * real_cost) {
@@ -1947,13 +1973,9 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
                 real_cost = c[0].first;
             }
         }
-        if (logn != P.tz32.logn && want != BATCH_PAIR && (want == BATCH_REAL || best < 0 || real_cost < best_cost))
-        {
-            free_tz(bt.tz);   // of a first call that failed later on
-            build_toeplitz<float>(P, bt.tz, logn + 1);
-            P.spec.clear();
-            P.spec_n = 0;
-        }
+        if (logn != P.tz32.logn && want != BATCH_PAIR && (want == BATCH_REAL || best < 0 || real_cost < best_cost) &&
+            !build_batch_real(P, logn))
+            real_cost = own_cost;
     }
     if (best < 0 && real_cost < 0.0) throw Error{MM_ERR_ARG, "lambda too large for the batched FFT blocks"};
     if ((want == BATCH_PAIR && best < 0) || (want == BATCH_REAL && real_cost < 0.0))

@@ -94,8 +94,9 @@ def dead(ls):
     return [l for l in ls if l[2] != 0]
 
 
-# (interval lengths, lambda, components): at 64 columns the pair form
-BATCHES = [([9000, 9000], 500, 3)]
+# (interval lengths, lambda, components): at 64 columns the pair form; the real form with the
+# plan's kind of block, and with one of the persistent kernel's, neither of them the plan's
+BATCHES = [([9000, 9000], 500, 3), ([40000, 40000], 500, 3), ([40000, 40000], 2000, 1)]
 
 
 @pytest.mark.parametrize("lengths,lam,ncomp", BATCHES)
