@@ -64,7 +64,7 @@ struct ToeplitzDev {
     void* ws_tab = nullptr;
     void* ws_H = nullptr;
     float* ws_scratch = nullptr;
-    void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N, folded (fold_split_spectra);
+    void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N (fold_split_spectra);
                              // FP32: T[npsd][N + 1], divided by another 4 (split_chain)
 };
 
@@ -253,8 +253,10 @@ bool symbol_positive(const std::vector<double>& t);
 std::vector<std::vector<double>> toeplitz_row_derivatives(double sigma, double fknee, double alpha, int64_t L,
                                                           double fsamp, int lam, int window);
 std::vector<double> overlap_save_spectrum(const std::vector<double>& t, int64_t N);
-// values of a folded spectrum: alpha [N], beta [N/2 + 1], one of padding
-__host__ __device__ constexpr int64_t split_size(int64_t N) { return N + N / 2 + 2; }
+// values of a folded spectrum: alpha [N], beta [N/2 + 1], sines [N/2 + 1], the number of chained
+// bins, one of padding
+__host__ __device__ constexpr int64_t split_size(int64_t N) { return 2 * N + 4; }
+constexpr double SPLIT_RATIO = 0.5;   // of H_k and H_{N-k}: below it a pair of bins is chained
 std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& spectra, int64_t N);
 // per-pass Stockham twiddles of an N = 2^logn point FFT as interleaved (cos, sin)
 std::vector<double> pass_twiddle_table(int logn);

@@ -69,7 +69,7 @@ struct TzArgs {
     const Tile* tiles;
     const T* twiddle;      // [N/2 + 1]: cos(2 pi k / B), cross-CTA step of the cluster blocks
     const typename Cx<T>::type* ptw;  // per-pass FFT twiddles (ptw_offset)
-    const T* H;            // [npsd][split_size(N)] folded spectra; FP32: [npsd][N + 1] spectra / 4
+    const T* H;            // [npsd][split_size(N)] (fold_split_spectra); FP32: [npsd][N + 1] spectra / 4
     const In<T>* y;        // time-domain input (mode 0)
     const double* yd;      // FP64 time-domain input (modes 2, 4, 5)
     const In<T>* x;        // map (gather modes)
@@ -702,12 +702,43 @@ __device__ __forceinline__ void store_out(const Tile& tile, In<T>* z, int lambda
 // Spectrum product of the packed real block at the bin pair (k, N - k), u1 = U_k, u2 =
 // U_{N-k}, returned conjugated: the forward FFT of conj(V) is conj of N * IFFT(V).
 //
-// FP64 and double-float: written out, the chain real-FFT split -> product with the real kernel
-// spectrum -> merge back to packed form is linear in u1 and conj(u2) with real coefficients
-// that depend on the kernel and k alone (fold_split_spectra):
+// split_chain: real-FFT split -> product with the real kernel spectrum -> merge back to packed
+// form.  h1 = H_k / 4, h2 = H_{N-k} / 4, (cw, sw) = (cos, sin) of pi k / N.
+template <typename T>
+__device__ __forceinline__ void split_chain(typename Cx<T>::type u1, typename Cx<T>::type u2, T cw, T sw, T h1, T h2,
+                                            typename Cx<T>::type& V1, typename Cx<T>::type& V2) {
+    using C2 = typename Cx<T>::type;
+    // twice E = (u1 + conj u2) / 2 and O = -i (u1 - conj u2) / 2
+    C2 E, O, Z1, Z2, S, D;
+    E.x = u1.x + u2.x; E.y = u1.y - u2.y;
+    O.x = u1.y + u2.y; O.y = u2.x - u1.x;
+    const C2 WO = cmul<T>(O, cw, sw);
+    // X_k = E + W O, conj X_{N-k} = E - W O, times the spectrum
+    Z1.x = h1 * (E.x + WO.x); Z1.y = h1 * (E.y + WO.y);
+    Z2.x = h2 * (E.x - WO.x); Z2.y = h2 * (E.y - WO.y);
+    // V_k = S + i conj(W) D, conj V_{N-k} = S - i conj(W) D
+    S.x = Z1.x + Z2.x; S.y = Z1.y + Z2.y;
+    D.x = Z1.x - Z2.x; D.y = Z1.y - Z2.y;
+    const T px = cw * D.x - sw * D.y, py = cw * D.y + sw * D.x;
+    V1.x = S.x - py; V1.y = -(S.y + px);
+    V2.x = S.x + py; V2.y = S.y - px;
+}
+
+// split_product: the same written out.  The chain is linear in u1 and conj(u2) with real
+// coefficients that depend on the kernel and k alone (fold_split_spectra):
 //   V_k = alpha_k u1 + i beta_k conj(u2),   V_{N-k} = alpha_{N-k} u2 + i beta_k conj(u1),
-// eight operations for the pair and no twiddle, where the chain took 44 (one A x in FP64 on
+// eight operations for the pair and no twiddle, where the chain takes 44 (one A x in FP64 on
 // 2^22 samples at lambda = 4096: 1.003 -> 0.924 ms, FP64-pipe bound).
+//
+// 1/f noise leaves H_k small at the low bins, where a map's time stream is largest.  The chain
+// multiplies the rounding errors of X_k by H_k; the folded form leaves them at the size of
+// H_{N-k} in both bins of the pair.  The error against 64 bits is the same in norm, but it sits in
+// the slow modes: FP32 PCG runs took 10 % more iterations on it, and of a smooth pulse at
+// f_knee = 1 to 2 Hz the FP64 product left 3e-15 to 1e-12 of the lowest modes as rounding, the
+// chain less than 2e-15.  So FP32 takes the chain throughout, FP64 and double-float for the
+// bins where H_k and H_{N-k} differ by more than a factor 1 / SPLIT_RATIO (f_knee = 2 Hz at 100
+// Hz: 1 bin in 12; A x of 2^22 I/Q/U samples 808 -> 813 us, the double-float residual
+// unchanged at 481).
 template <typename T>
 __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename Cx<T>::type u2, T a1, T a2, T b,
                                               typename Cx<T>::type& V1, typename Cx<T>::type& V2) {
@@ -717,27 +748,30 @@ __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename 
     V2.y = -(a2 * u2.y + b * u1.x);
 }
 
-// FP32: the chain itself.  1/f noise leaves H_k small at the low bins, where a map's time
-// stream is largest; the chain multiplies the rounding errors of X_k by H_k, the folded form
-// leaves them at full size in both bins of the pair.  The error against 64 bits is the same
-// in norm, but it sits in the slow modes: FP32 PCG runs took 10 % more iterations on it.
-// h1 = H_k / 4, h2 = H_{N-k} / 4, (cw, sw) = (cos, sin) of pi k / N.
-__device__ __forceinline__ void split_chain(float2 u1, float2 u2, float cw, float sw, float h1, float h2, float2& V1,
-                                            float2& V2) {
-    // twice E = (u1 + conj u2) / 2 and O = -i (u1 - conj u2) / 2
-    const float2 E = make_float2(u1.x + u2.x, u1.y - u2.y);
-    const float2 O = make_float2(u1.y + u2.y, u2.x - u1.x);
-    const float2 WO = cmul<float>(O, cw, sw);
-    // X_k = E + W O, conj X_{N-k} = E - W O, times the spectrum
-    const float2 Z1 = make_float2(h1 * (E.x + WO.x), h1 * (E.y + WO.y));
-    const float2 Z2 = make_float2(h2 * (E.x - WO.x), h2 * (E.y - WO.y));
-    // V_k = S + i conj(W) D, conj V_{N-k} = S - i conj(W) D
-    const float2 S = make_float2(Z1.x + Z2.x, Z1.y + Z2.y);
-    const float2 D = make_float2(Z1.x - Z2.x, Z1.y - Z2.y);
-    const float px = cw * D.x - sw * D.y, py = cw * D.y + sw * D.x;
-    V1 = make_float2(S.x - py, -(S.y + px));
-    V2 = make_float2(S.x + py, S.y - px);
-}
+// A row of fold_split_spectra (FP64, double-float): the product of bins k and N - k, k < N, with
+// a1 = alpha_k and a2 = alpha_{N-k} (alpha_0 for k = 0) read ahead by the caller.
+template <typename T, int N>
+struct SplitRow {
+    const T *al, *be, *si;
+    int kc;
+    __device__ __forceinline__ explicit SplitRow(const T* row) : al(row), be(row + N), si(row + N + N / 2 + 1) {
+        const T v = si[N / 2 + 1];
+        if constexpr (std::is_same<T, double>::value) kc = (int)v;
+        else kc = (int)v.hi;
+    }
+    __device__ __forceinline__ void product(typename Cx<T>::type u1, typename Cx<T>::type u2, int k, T a1, T a2,
+                                            typename Cx<T>::type& V1, typename Cx<T>::type& V2) const {
+        const int m = k <= N / 2 ? k : N - k;
+        const T b = be[m];
+        if (m < kc) {
+            const T sw = si[m];
+            if (k == 0) split_chain<T>(u1, u2, (T)1.0, sw, a1, b, V1, V2);
+            else split_chain<T>(u1, u2, k <= N / 2 ? b : -b, sw, a1, a2, V1, V2);
+        } else {
+            split_product<T>(u1, u2, a1, a2, b, V1, V2);
+        }
+    }
+};
 
 template <typename T, int LOGN, int NT, int MODE>
 __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
@@ -768,7 +802,7 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
             float sw, cw;
             sincospif((float)k * (1.f / (float)N), &sw, &cw);
             C2 V1, V2;
-            split_chain(a[pad<T>(k)], a[pad<T>(k2)], cw, sw, h1, h2, V1, V2);
+            split_chain<T>(a[pad<T>(k)], a[pad<T>(k2)], cw, sw, h1, h2, V1, V2);
             a[pad<T>(k)] = V1;
             if (k2 != k) a[pad<T>(k2)] = V2;
         };
@@ -786,13 +820,11 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
         }
         if (tid == 0) product(N / 2, __ldg(H + N / 2), __ldg(H + N / 2));
     } else {
-        constexpr int64_t HS = split_size(N);
-        const T* al = A.H + tile.psd * HS;
-        const T* be = al + N;
+        const SplitRow<T, N> row(A.H + tile.psd * split_size(N));
         for (int k = tid; k <= N / 2; k += NT) {
             const int k2 = (N - k) & (N - 1);
             C2 V1, V2;
-            split_product<T>(a[pad<T>(k)], a[pad<T>(k2)], al[k], al[k2], be[k], V1, V2);
+            row.product(a[pad<T>(k)], a[pad<T>(k2)], k, row.al[k], row.al[k2], V1, V2);
             a[pad<T>(k)] = V1;
             if (k2 != k) a[pad<T>(k2)] = V2;
         }
@@ -917,16 +949,16 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int64_t HS = F32 ? N + 1 : split_size(N);
     const T* al = A.H + tile.psd * HS;
-    const T* be = al + N;
     // bins k and N - k (FP32: the chain, al = the spectrum itself, h1 and h2 its values)
+    using Row = typename std::conditional<F32, const T*, SplitRow<T, N>>::type;
+    const Row row(al);
     auto product = [&](C2 u1, C2 u2, int k, T h1, T h2, C2& V1, C2& V2) {
         if constexpr (F32) {
             float sw, cw;
             sincospif((float)k * (1.f / (float)N), &sw, &cw);
-            split_chain(u1, u2, cw, sw, h1, h2, V1, V2);
+            split_chain<T>(u1, u2, cw, sw, h1, h2, V1, V2);
         } else {
-            const int k2 = (N - k) & (N - 1);
-            split_product<T>(u1, u2, h1, h2, be[k < k2 ? k : k2], V1, V2);
+            row.product(u1, u2, k, h1, h2, V1, V2);
         }
     };
     auto second = [&](int k) { return F32 ? N - k : (N - k) & (N - 1); };   // index of h2

@@ -544,7 +544,7 @@ __device__ __forceinline__ void chain2(cx2& u1, cx2& u2, cx2 w, f2 h1, f2 h2) {
 // the same for one pair
 __device__ __forceinline__ void chain1(float2& u1, float2& u2, float2 w, float h1, float h2) {
     float2 V1, V2;
-    split_chain(u1, u2, w.x, -w.y, h1, h2, V1, V2);
+    split_chain<float>(u1, u2, w.x, -w.y, h1, h2, V1, V2);
     u1 = make_float2(V1.x, -V1.y);
     u2 = make_float2(V2.x, -V2.y);
 }
