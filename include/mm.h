@@ -159,16 +159,17 @@ mm_status mm_scatter_config(mm_plan_t plan, int32_t* lanes_per_pixel, float* ms)
  *         0: two right-hand sides per complex FFT of 2^log2_block points (real kernel
  *         spectrum: real and imaginary parts convolve independently);
  *         1: one real FFT per right-hand side, with the FP32 block of mm_plan_info or (where
- *         neither that block nor autotuning was asked for) one better for R of them;
+ *         neither that block nor autotuning was asked for) one better for R of them, which
+ *         depends on R alone: a call on R columns gives the same after any other calls;
  *         2: the band product as a dense contraction on the tensor cores (tcgen05 MMAs in
  *         FP16 on operands split as hi + 2^-11 lo after power-of-two scaling, FP32
  *         accumulators in tensor memory; 128-row tiles, window 128 + 2 lambda; the maps
  *         are de-pointed into a [R][nt] buffer first); log2_block reports 7 (the tile).
  *         Choosing times all three forms at R columns when the plan autotunes, else takes
- *         the cheaper FFT form by the cost model (the contraction costs 2 (2 lambda + 128)
- *         flops per sample and column against ~10 log2 B for the FFT).  Asking for a form
- *         other than the fixed one, or one that no block supports for this lambda, is
- *         MM_ERR_ARG.
+ *         the cheaper FFT form by the cost model for 64 columns (the contraction costs
+ *         2 (2 lambda + 128) flops per sample and column against ~10 log2 B for the FFT).
+ *         Asking for a form other than the fixed one, or one that no block supports for this
+ *         lambda, is MM_ERR_ARG.
  *   R     1..64, the column count for the timing (and the buffers it allocates).
  *   log2_block, ms (host float[3]: timed launches of forms 0, 1 and 2, or 0): may be NULL.
  */

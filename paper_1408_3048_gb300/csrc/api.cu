@@ -129,7 +129,10 @@ enum { BATCH_PAIR = 0, BATCH_REAL = 1, BATCH_TENSOR = 2 };
 struct BatchState {
     int kind = -1;                // BATCH_PAIR / BATCH_REAL / BATCH_TENSOR, -1 before the first call
     float tuned_ms[3] = {};       // timed forms (autotuning), 0 when not timed
-    ToeplitzDev tz;               // real form: its own FP32 block, where the plan's is not the best for R
+    // real form: FP32 blocks by logn, built when a call's columns take another one than the plan's,
+    // and the block for R columns (0: not asked for yet)
+    ToeplitzDev tz[20];
+    signed char real_logn[BATCH_RMAX + 1] = {};
     int logb = 0;                 // complex FFT length of the pair kernel
     int ntiles = 0;
     SpanTile* tiles = nullptr;
@@ -242,7 +245,7 @@ static void destroy_plan(PlanHolder* P) {
     }
     for (auto e : P->prof.pool) (void)cudaEventDestroy(e);
     BatchState& bt = P->batch;
-    free_tz(bt.tz);
+    for (ToeplitzDev& t : bt.tz) free_tz(t);
     if (bt.graph) (void)cudaGraphExecDestroy(bt.graph);
     for (void* p : {(void*)bt.tiles, (void*)bt.H, (void*)bt.ptw, (void*)bt.twiddle, (void*)bt.x, (void*)bt.r,
                     (void*)bt.p, (void*)bt.q, (void*)bt.z,
@@ -1780,6 +1783,9 @@ static void grad(PlanHolder& P, const double* d, const double* m, const double* 
 // Complex-pair kernel tables for a 2^logb-point block.
 static void build_batch_pair(PlanHolder& P, int logb) {
     BatchState& bt = P.batch;
+    for (void* p : {(void*)bt.tiles, (void*)bt.H, (void*)bt.ptw, (void*)bt.twiddle}) dfree(p);   // of a build that failed
+    bt.tiles = nullptr;
+    bt.H = bt.ptw = bt.twiddle = nullptr;
     bt.logb = logb;
     const int64_t B = int64_t(1) << logb;
     const int64_t Lv = B - 2 * (int64_t)P.lambda;
@@ -1894,45 +1900,75 @@ static void ensure_batch_tc_buffer(PlanHolder& P, int R) {
 }
 
 static void launch_batch_tz(PlanHolder& P, int R, const float* X, float* Z, const int* done);
-static const ToeplitzDev& batch_tz(const PlanHolder& P) { return P.batch.tz.logn != 0 ? P.batch.tz : P.tz32; }
 
-// The real form's own block, complete or (false) not at all: without memory for it the plan's
-// block serves.
-static bool build_batch_real(PlanHolder& P, int logn) {
+// The real form's block for R right-hand sides: one that fills the chip with R launches' worth
+// of tiles can be larger than the one with the shortest single launch.  It depends on R alone,
+// not on the calls before.
+static int batch_real_logn(PlanHolder& P, int R) {
+    signed char& l = P.batch.real_logn[R];
+    if (l == 0) {
+        l = (signed char)P.tz32.logn;
+        if (!P.forced_f32 && !P.autotune) {
+            const auto c = block_candidates<float>(P, R);
+            if (c[0].first < 0.95 * block_us<float>(P, P.tz32.logn, (int64_t)P.tz32.ntiles * R)) l = (signed char)c[0].second;
+        }
+    }
+    return l;
+}
+
+// Block of an FP32 launch over R columns: in the real form the one for R, where it is built
+// (ensure_batch_real).
+static const ToeplitzDev& batch_tz(const PlanHolder& P, int R) {
+    const ToeplitzDev& t = P.batch.tz[P.batch.real_logn[R]];
+    return P.batch.kind == BATCH_REAL && t.logn != 0 ? t : P.tz32;
+}
+
+// Builds the real form's block for R columns, completely or not at all: without memory for it
+// the plan's block serves.
+static void ensure_batch_real(PlanHolder& P, int R) {
+    BatchState& bt = P.batch;
+    const int logn = batch_real_logn(P, R);
+    if (logn == P.tz32.logn || bt.tz[logn].logn != 0) return;
     ToeplitzDev t;
-    bool ok = false;
+    mm_status st = MM_OK;
     try {
         build_toeplitz<float>(P, t, logn + 1);
-        ok = true;
     } catch (const Error& e) {
-        if (e.st != MM_ERR_OOM) {
-            free_tz(t);
-            throw;
-        }
+        st = e.st;
+        free_tz(t);
+        if (st != MM_ERR_OOM) throw;
     } catch (...) {
         free_tz(t);
         throw;
     }
     P.spec.clear();
     P.spec_n = 0;
-    if (!ok) free_tz(t);
-    else P.batch.tz = t;
-    return ok;
+    if (st != MM_OK) return;
+    bt.tz[logn] = t;
+    if (bt.graph) {   // it may hold launches on the plan's block
+        (void)cudaGraphExecDestroy(bt.graph);
+        bt.graph = nullptr;
+    }
 }
 
 // Batched Toeplitz form, chosen once per plan (before any graph capture), after the
 // R-column buffers exist:
 //   BATCH_PAIR  two RHS per complex FFT (y_a + i y_b, one complex block of 2^logb points,
 //               block > 2 lambda complex points);
-//   BATCH_REAL  the single-RHS real-FFT kernel with an RHS grid dimension (its FP32
-//               block, B > 2 lambda reals, so half the FFT length of the pair form).
+//   BATCH_REAL  the single-RHS real-FFT kernel with an RHS grid dimension (FP32 blocks,
+//               B > 2 lambda reals, so half the FFT length of the pair form).
 // Cost model: block_us of the real form's tiles, and for the pair form its operation count at
-// a measured rate; ties go to the pair form.  With autotuning both are timed at this R.
+// a measured rate, both for BATCH_RMAX columns, so that the first call's number does not
+// matter (the real form is as fast or faster at fewer: 2^22 I/Q/U samples at lambda = 1024,
+// R = 64 1850 against 2159 us, R = 1 157 against 194; where the pair form is ahead at 64
+// columns, T, 2 x 18000 samples at lambda = 500, it is at one, 42 against 45); ties go to the
+// pair form.  With autotuning all forms are timed at this R.
 static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
     BatchState& bt = P.batch;
     if (bt.kind >= 0) {
         if (want >= 0 && want != bt.kind) throw Error{MM_ERR_ARG, "the batched form is already fixed"};
         if (bt.kind == BATCH_TENSOR) ensure_batch_tc_buffer(P, R);
+        if (bt.kind == BATCH_REAL) ensure_batch_real(P, R);
         return;
     }
     if (want == BATCH_TENSOR) {
@@ -1951,31 +1987,17 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
         // two right-hand sides per transform; SM time per operation measured at lambda = 1024
         // .. 16384, the cluster blocks' relative to it
         const double weight = cl == 4 ? 3.3 : (cl == 2 ? 1.6 : 1.0);
-        const double us = (double)interval_tiles(P, Lv) * ((R + 1) / 2) * ((double)B * logb + 2048.0) * weight * 1.28e-4;
+        const double us = (double)interval_tiles(P, Lv) * (BATCH_RMAX / 2) * ((double)B * logb + 2048.0) * weight * 1.28e-4;
         const double cost = std::max(15.0, us / P.num_sms);
         if (best < 0 || cost < best_cost) {
             best = logb;
             best_cost = cost;
         }
     }
-    // the real form's block for this many right-hand sides: one that fills the chip with R
-    // launches' worth of tiles can be larger than the one with the shortest single launch
-    free_tz(bt.tz);   // of a first call that failed later on
     double real_cost = -1.0;
     if (P.tz32.logn != 0) {
-        const double own_cost = block_us<float>(P, P.tz32.logn, (int64_t)P.tz32.ntiles * R);
-        int logn = P.tz32.logn;
-        real_cost = own_cost;
-        if (!P.forced_f32 && !P.autotune) {
-            const auto c = block_candidates<float>(P, R);
-            if (c[0].first < 0.95 * real_cost) {
-                logn = c[0].second;
-                real_cost = c[0].first;
-            }
-        }
-        if (logn != P.tz32.logn && want != BATCH_PAIR && (want == BATCH_REAL || best < 0 || real_cost < best_cost) &&
-            !build_batch_real(P, logn))
-            real_cost = own_cost;
+        const int logn = batch_real_logn(P, BATCH_RMAX);
+        real_cost = block_us<float>(P, logn, overlap_tiles(P, logn) * BATCH_RMAX);
     }
     if (best < 0 && real_cost < 0.0) throw Error{MM_ERR_ARG, "lambda too large for the batched FFT blocks"};
     if ((want == BATCH_PAIR && best < 0) || (want == BATCH_REAL && real_cost < 0.0))
@@ -2017,6 +2039,7 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
     } else {
         bt.kind = best_cost <= real_cost ? BATCH_PAIR : BATCH_REAL;
     }
+    if (bt.kind == BATCH_REAL) ensure_batch_real(P, R);
 }
 
 static void ensure_batch_buffers(PlanHolder& P, int R) {
@@ -2074,7 +2097,7 @@ static BatchTzArgs batch_tz_args(PlanHolder& P, int R, const float* X, float* Z,
 static void launch_batch_tz(PlanHolder& P, int R, const float* X, float* Z, const int* done) {
     BatchState& bt = P.batch;
     if (bt.kind == BATCH_REAL) {
-        launch_toeplitz_rhs<float>(P, batch_tz(P), nullptr, X, R, P.n, Z, P.nt, done, P.stream);
+        launch_toeplitz_rhs<float>(P, batch_tz(P, R), nullptr, X, R, P.n, Z, P.nt, done, P.stream);
     } else if (bt.kind == BATCH_TENSOR) {
         // column scales from the maps, Y = P X, then the band product on the tensor cores
         launch_batch_colscale(X, P.n, R, bt.tc_scale, bt.tc_scale + BATCH_RMAX, P.stream);
@@ -2231,7 +2254,6 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
         throw Error{MM_ERR_ARG, "the batched solver runs MM_SOLVE_MIXED with MM_PREC_BD"};
     const int RB = std::min(R, BATCH_RMAX);
     ensure_batch_buffers(P, RB);
-    ensure_batch_tables(P, RB);
     BatchState& bt = P.batch;
     const bool d_dev = is_device_ptr(D), m_dev = is_device_ptr(M);
     const size_t n = (size_t)P.n, nt = (size_t)P.nt;
@@ -2240,6 +2262,7 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
     int overall = MM_OK;
     for (int c0 = 0; c0 < R; c0 += RB) {
         const int Rc = std::min(RB, R - c0);
+        ensure_batch_tables(P, Rc);
         check_cuda(cudaEventRecord(P.ev0, s), "event");
         std::vector<double> bb(Rc), rr(Rc);
         std::vector<int> iters(Rc, 0), outer(Rc, 0), fp64(Rc, 0);
@@ -2256,7 +2279,7 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
         // b_r = P^T N^-1 d_r in FP32 for all columns in one batched Toeplitz launch (it seeds
         // the first inner solve and scales the residual; the FP64 residuals come from the
         // data, residual64)
-        launch_toeplitz_any<float>(P, batch_tz(P), nullptr, Dg, nullptr, Rc, (int64_t)nt, bt.tod, (int64_t)nt, nullptr, s);
+        launch_toeplitz_any<float>(P, batch_tz(P, Rc), nullptr, Dg, nullptr, Rc, (int64_t)nt, bt.tod, (int64_t)nt, nullptr, s);
         launch_batch_scatter(P, bt.tod, bt.z, Rc, nullptr, s);
         launch_convert_f32_to_f64(bt.z, bt.b64, (int64_t)Rc * n, s);
         launch_dot_batch(bt.b64, (int64_t)n, Rc, bt.scal, s);
@@ -2737,7 +2760,7 @@ mm_status mm_batch_config(mm_plan_t plan, int32_t R, int32_t* kind, int32_t* log
         sync(*P);
         const BatchState& bt = P->batch;
         *kind = bt.kind;
-        if (log2_block) *log2_block = bt.kind == BATCH_REAL ? batch_tz(*P).logn + 1 : (bt.kind == BATCH_TENSOR ? 7 : bt.logb);
+        if (log2_block) *log2_block = bt.kind == BATCH_REAL ? batch_tz(*P, R).logn + 1 : (bt.kind == BATCH_TENSOR ? 7 : bt.logb);
         if (ms) {
             ms[0] = bt.tuned_ms[0];
             ms[1] = bt.tuned_ms[1];

@@ -120,3 +120,23 @@ def test_batched_call_without_memory(lib, lengths, lam, ncomp):
         if done:
             break
     assert failed >= 17 and done
+
+
+@pytest.mark.parametrize("lengths,lam,ncomp", BATCHES + [([300000, 300000], 1024, 3), ([131072], 1024, 1)])
+def test_batched_call_does_not_depend_on_the_calls_before(lib, lengths, lam, ncomp):
+    """Form, block and launches of R columns are those of a fresh plan, whatever R came first."""
+    def fresh(R):
+        p = Plan(lib, lengths, lam, ncomp)
+        out = p.batch(R), p.solve_batch(R)
+        cfg = p.config(R)
+        p.close()
+        return out, cfg
+
+    Rs = [1, 2, 7, 16, 64]
+    want = {R: fresh(R) for R in Rs}
+    for order in (Rs, Rs[::-1]):
+        p = Plan(lib, lengths, lam, ncomp)
+        for R in order:
+            assert (p.batch(R), p.solve_batch(R)) == want[R][0], (order[0], R)
+            assert p.config(R) == want[R][1]
+        p.close()
