@@ -203,7 +203,6 @@ static void free_tz(ToeplitzDev& t) {
     dfree(t.H);
     dfree(t.ws_tab);
     dfree(t.ws_H);
-    dfree(t.ws_scratch);
     t = ToeplitzDev{};
 }
 
@@ -223,7 +222,7 @@ static void destroy_plan(PlanHolder* P) {
                     (void*)P->sl_w64, (void*)P->sl_w32, (void*)P->sl_ang, (void*)P->ioff, (void*)P->ipsd, (void*)P->t0,
                     (void*)P->bd64, (void*)P->bd32, (void*)P->tod64, (void*)P->tod32, (void*)P->map4, (void*)P->dbuf,
                     (void*)P->b64, (void*)P->d_dot, (void*)P->x64, (void*)P->r64, (void*)P->ax64,
-                    (void*)P->grad_H, (void*)P->grad_u, (void*)P->grad_part})
+                    (void*)P->grad_H, (void*)P->grad_u, (void*)P->grad_part, (void*)P->ws_scratch})
         dfree(p);
     free_tz(P->tz64);
     free_tz(P->tz32);
@@ -463,7 +462,8 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
             h2d(tz.ws_tab, tab.data(), tab.size() * 4, P.stream);
             tz.ws_H = dalloc<float>(Hw.size());
             h2d(tz.ws_H, Hw.data(), Hw.size() * 4, P.stream);
-            tz.ws_scratch = dalloc<float>(ws_scratch_floats(tz.logn, P.num_sms));
+            if (P.ws_scratch == nullptr) P.ws_scratch = dalloc<float>(ws_scratch_floats(P.num_sms));
+            tz.ws_scratch = P.ws_scratch;
             sync(P.stream);
             return;
         }

@@ -59,8 +59,8 @@ struct ToeplitzDev {
     Tile* tiles = nullptr;   // [ntiles]
     void* twiddle = nullptr; // T[B/4 + 1]: cos(2 pi k / B) (cluster blocks)
     void* ptw = nullptr;     // T2[...]: per-pass twiddles of the N-point FFT (not FP32)
-    // FP32 blocks of 2^14 and 2^15 reals (toeplitz_ws.cu): twiddle tables, folded spectra in
-    // the kernel's order, and two input buffers of B floats per resident CTA
+    // FP32 blocks of 2^14 and 2^15 reals (toeplitz_ws.cu): twiddle tables, spectra in the kernel's
+    // order, and the plan's input buffers
     void* ws_tab = nullptr;
     void* ws_H = nullptr;
     float* ws_scratch = nullptr;
@@ -166,6 +166,7 @@ struct Plan {
     double* t0 = nullptr;          // [npsd] diagonal of each row
 
     ToeplitzDev tz64, tz32;
+    float* ws_scratch = nullptr;   // input buffers of the persistent kernel (toeplitz_ws.cu), or null
     ToeplitzDev tzdf;              // double-float tables (refinement residual)
     std::vector<std::vector<double>> spec;   // spectra of the rows while tables are built (N = spec_n)
     int64_t spec_n = 0;
@@ -290,7 +291,7 @@ void launch_toeplitz_f32_packed(const Plan& P, const float* x, bool pack, float*
 bool ws_supported(int logn);
 std::vector<float> ws_tables(int logn);
 std::vector<float> ws_spectra(const std::vector<std::vector<double>>& spectra, int logn);
-size_t ws_scratch_floats(int logn, int num_sms);
+size_t ws_scratch_floats(int num_sms);
 template <typename T>
 size_t toeplitz_smem_bytes(int logn);
 template <typename T>

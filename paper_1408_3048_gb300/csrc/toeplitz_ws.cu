@@ -795,7 +795,9 @@ bool ws_supported(int logn) { return logn == 13 || logn == 14; }
 
 // CTAs launched at most: the resident ones (one of 2^15 reals, two of 2^14, per SM)
 static int ws_ctas(int logn, int num_sms) { return num_sms << (14 - logn); }
-size_t ws_scratch_floats(int logn, int num_sms) { return (size_t)ws_ctas(logn, num_sms) * 2 * (size_t(2) << logn); }
+// Two buffers of B floats per CTA: 262 KB per SM for either block.  One set per plan: all of
+// its launches, of its own block and the batch's, run one after the other on its stream.
+size_t ws_scratch_floats(int num_sms) { return (size_t)ws_ctas(14, num_sms) * 2 * (size_t(2) << 14); }
 
 template <int LOGN>
 static void ws_launch(const TzArgs<float>& A, const ToeplitzDev& tz, int num_sms, int mode, cudaStream_t s) {

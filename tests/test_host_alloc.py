@@ -140,3 +140,16 @@ def test_batched_call_does_not_depend_on_the_calls_before(lib, lengths, lam, nco
             assert (p.batch(R), p.solve_batch(R)) == want[R][0], (order[0], R)
             assert p.config(R) == want[R][1]
         p.close()
+
+
+def test_one_set_of_input_buffers_per_plan(lib):
+    """The persistent kernel's input buffers (two of 2^15 floats per SM) are the plan's: a plan whose
+    batch has a block of its own, both of that kernel, holds one set as a plan with one block."""
+    buffers, held = 152 * 2 * (1 << 15) * 4, []
+    for log2_f32, block in ((0, 1 << 14), (15, 1 << 15)):
+        before = lib.fake_live_bytes()
+        p = Plan(lib, [300000, 300000], 4000, 1, fft_log2_f32=log2_f32)
+        assert p.block32 == block and p.config(8) == (1, 15)
+        held.append(lib.fake_live_bytes() - before)
+        p.close()
+    assert buffers < held[0] < held[1] + buffers // 8
