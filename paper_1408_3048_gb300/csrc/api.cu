@@ -413,20 +413,41 @@ static int choose_logn(const Plan& P, int forced_log2B, int* cluster) {
     return logn;
 }
 
-// Overlap-save spectra of the plan's rows for N-point blocks.  The grid of a smaller block is
+// Overlap-save spectrum of row p of the plan for N-point blocks.  The grid of a smaller block is
 // a subset of a larger one's, so the transforms of the largest block asked for so far are kept
-// while the plan is built (three arithmetics ask, often for different blocks).
-static std::vector<std::vector<double>> plan_spectra(Plan& P, int64_t N) {
+// while the plan is built (three arithmetics ask, often for different blocks), where they take
+// no more than 64 MB; plans of many PSDs transform each row when it is asked for.
+static std::vector<double> plan_spectrum(Plan& P, int p, int64_t N) {
     if (P.spec_n < N) {
+        if ((int64_t)P.npsd * (N + 1) * 8 > (int64_t(64) << 20)) return overlap_save_spectrum(P.rows[(size_t)p], N);
         P.spec_n = N;
         P.spec.clear();
         for (const auto& r : P.rows) P.spec.push_back(overlap_save_spectrum(r, N));
     }
     const int64_t step = P.spec_n / N;
-    std::vector<std::vector<double>> out((size_t)P.npsd, std::vector<double>((size_t)N + 1));
-    for (int p = 0; p < P.npsd; ++p)   // (the spectra are divided by their own N)
-        for (int64_t k = 0; k <= N; ++k) out[(size_t)p][(size_t)k] = P.spec[(size_t)p][(size_t)(k * step)] * (double)step;
+    std::vector<double> out((size_t)N + 1);
+    for (int64_t k = 0; k <= N; ++k)   // (the spectra are divided by their own N)
+        out[(size_t)k] = P.spec[(size_t)p][(size_t)(k * step)] * (double)step;
     return out;
+}
+
+// Rows of fold_split_spectrum in T on the device, [kinds][rows]; spectrum(row, kind) is asked for
+// every kind of a row in turn.
+template <typename T, typename F>
+static T* fold_rows(Plan& P, int kinds, int rows, int64_t N, F&& spectrum) {
+    const std::vector<double> quarter = quarter_wave(2 * N);
+    std::vector<double> row((size_t)split_size(N));
+    std::vector<T> H((size_t)kinds * rows * row.size());
+    for (int p = 0; p < rows; ++p)
+        for (int c = 0; c < kinds; ++c) {
+            fold_split_spectrum(spectrum(p, c), N, quarter, row.data());
+            T* h = H.data() + ((size_t)c * rows + p) * row.size();
+            for (size_t i = 0; i < row.size(); ++i) h[i] = T(row[i]);
+        }
+    std::unique_ptr<T, void (*)(T*)> dev(dalloc<T>(H.size()), [](T* q) { dfree(q); });
+    h2d(dev.get(), H.data(), H.size() * sizeof(T), P.stream);
+    sync(P.stream);   // host vectors go out of scope
+    return dev.release();
 }
 
 template <typename T>
@@ -438,9 +459,9 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
     tz.ntiles = (int)tiles.size();
     tz.tiles = dalloc<Tile>(tiles.size());
     h2d(tz.tiles, tiles.data(), tiles.size() * sizeof(Tile), P.stream);
-    if (tz.cluster > 1) {   // cross-CTA twiddles
-        std::vector<T> tw((size_t)(B / 4 + 1));
-        for (int64_t k = 0; k <= B / 4; ++k) tw[(size_t)k] = (T)std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B);
+    if (sizeof(T) == 8 || tz.cluster > 1) {   // cross-CTA twiddles, chained bins of FP64
+        const std::vector<double> quarter = quarter_wave(B);
+        const std::vector<T> tw(quarter.begin(), quarter.end());
         tz.twiddle = dalloc<T>(tw.size());
         h2d(tz.twiddle, tw.data(), tw.size() * sizeof(T), P.stream);
         sync(P.stream);
@@ -454,31 +475,28 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
         h2d(tz.ptw, ptT.data(), ptT.size() * sizeof(T), P.stream);
         sync(P.stream);
     }
-    const std::vector<std::vector<double>> spec = plan_spectra(P, N);
+    auto spectrum = [&](int p, int) { return plan_spectrum(P, p, N); };
     if constexpr (sizeof(T) == 4) {
+        std::vector<float> H;
         if (tz.cluster == 1 && ws_supported(tz.logn)) {
-            const std::vector<float> tab = ws_tables(tz.logn), Hw = ws_spectra(spec, tz.logn);
+            const std::vector<float> tab = ws_tables(tz.logn);
             tz.ws_tab = dalloc<float>(tab.size());
             h2d(tz.ws_tab, tab.data(), tab.size() * 4, P.stream);
-            tz.ws_H = dalloc<float>(Hw.size());
-            h2d(tz.ws_H, Hw.data(), Hw.size() * 4, P.stream);
+            for (int p = 0; p < P.npsd; ++p) ws_append_spectrum(spectrum(p, 0), tz.logn, H);
+            tz.ws_H = dalloc<float>(H.size());
+            h2d(tz.ws_H, H.data(), H.size() * 4, P.stream);
             if (P.ws_scratch == nullptr) P.ws_scratch = dalloc<float>(ws_scratch_floats(P.num_sms));
             tz.ws_scratch = P.ws_scratch;
-            sync(P.stream);
-            return;
+        } else {
+            for (int p = 0; p < P.npsd; ++p)
+                for (double v : spectrum(p, 0)) H.push_back((float)(0.25 * v));
+            tz.H = dalloc<float>(H.size());
+            h2d(tz.H, H.data(), H.size() * sizeof(T), P.stream);
         }
-    }
-    std::vector<T> H;
-    if constexpr (sizeof(T) == 4) {
-        for (const auto& h : spec)
-            for (double v : h) H.push_back((T)(0.25 * v));
+        sync(P.stream);   // host vectors go out of scope
     } else {
-        const std::vector<double> Hd = fold_split_spectra(spec, N);
-        H.assign(Hd.begin(), Hd.end());
+        tz.H = fold_rows<T>(P, 1, P.npsd, N, spectrum);
     }
-    tz.H = dalloc<T>(H.size());
-    h2d(tz.H, H.data(), H.size() * sizeof(T), P.stream);
-    sync(P.stream);   // host vectors go out of scope
 }
 
 // Double-float tables (where the FP64 kernel has a block): the cosine and per-pass twiddles
@@ -498,24 +516,18 @@ static void build_toeplitz_df(Plan& P, int forced_log2B) {
         tz.tiles = dalloc<Tile>(tiles.size());
         h2d(tz.tiles, tiles.data(), tiles.size() * sizeof(Tile), P.stream);
         sync(P.stream);
-        std::vector<dfl> tw(tz.cluster > 1 ? (size_t)(B / 4 + 1) : 1);
-        if (tz.cluster > 1) {   // cross-CTA twiddles
-            for (int64_t k = 0; k <= B / 4; ++k) tw[(size_t)k] = dfl(std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B));
-            tz.twiddle = dalloc<dfl>(tw.size());
-            h2d(tz.twiddle, tw.data(), tw.size() * sizeof(dfl), P.stream);
-        }
+        std::vector<dfl> tw;   // cross-CTA twiddles, chained bins
+        for (double v : quarter_wave(B)) tw.push_back(dfl(v));
+        tz.twiddle = dalloc<dfl>(tw.size());
+        h2d(tz.twiddle, tw.data(), tw.size() * sizeof(dfl), P.stream);
         const int lc = tz.cluster == 4 ? 2 : (tz.cluster == 2 ? 1 : 0);
         const std::vector<double> pt = pass_twiddle_table(tz.logn - lc);
         std::vector<dfl> ptd(pt.size());
         for (size_t i = 0; i < pt.size(); ++i) ptd[i] = dfl(pt[i]);
         tz.ptw = dalloc<dfl>(ptd.size());
         h2d(tz.ptw, ptd.data(), ptd.size() * sizeof(dfl), P.stream);
-        const std::vector<double> Hd = fold_split_spectra(plan_spectra(P, N), N);
-        std::vector<dfl> H(Hd.size());
-        for (size_t i = 0; i < Hd.size(); ++i) H[i] = dfl(Hd[i]);
-        tz.H = dalloc<dfl>(H.size());
-        h2d(tz.H, H.data(), H.size() * sizeof(dfl), P.stream);
         sync(P.stream);   // host vectors go out of scope
+        tz.H = fold_rows<dfl>(P, 1, P.npsd, N, [&](int p, int) { return plan_spectrum(P, p, N); });
     } catch (...) {
         free_tz(tz);
         tz = ToeplitzDev{};
@@ -821,7 +833,7 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
             } catch (const Error&) {   // reported by the build below
             }
         }
-        if (logn > 0) (void)plan_spectra(P, int64_t(1) << logn);
+        if (logn > 0) (void)plan_spectrum(P, 0, int64_t(1) << logn);
     }
     // A precision whose largest block cannot hold the band is left unbuilt (logn = 0):
     // its operators then fail with MM_ERR_ARG; at least one precision must exist.
@@ -1697,21 +1709,17 @@ static void ensure_grad(PlanHolder& P) {
     if (P.grad_H != nullptr) return;
     if (P.tz64.logn == 0) throw Error{MM_ERR_ARG, "the PSD gradient needs an FP64 Toeplitz block for this lambda"};
     const int64_t N = int64_t(1) << P.tz64.logn;
-    std::vector<std::vector<double>> rows((size_t)3 * P.npsd);
-    for (int p = 0; p < P.npsd; ++p) {
+    for (int p = 0; p < P.npsd; ++p)
         if (!(P.h_psd[(size_t)p].fknee > 0.0)) throw Error{MM_ERR_ARG, "the PSD gradient needs fknee > 0"};
-        const auto D = toeplitz_row_derivatives(P.h_psd[(size_t)p].sigma, P.h_psd[(size_t)p].fknee,
-                                                P.h_psd[(size_t)p].alpha, P.L_grid, P.fsamp, P.lambda, P.window);
-        for (int c = 0; c < 3; ++c) rows[(size_t)c * P.npsd + p] = D[(size_t)c];
-    }
-    std::vector<std::vector<double>> spec;
-    for (const auto& r : rows) spec.push_back(overlap_save_spectrum(r, N));
-    const std::vector<double> H = fold_split_spectra(spec, N);
-    P.grad_H = dalloc<double>(H.size());
-    h2d(P.grad_H, H.data(), H.size() * 8, P.stream);
-    P.grad_u = dalloc<double>((size_t)P.nt);
-    P.grad_part = dalloc<double>((size_t)P.K);
-    sync(P.stream);
+    // the vectors first: the spectra are the sign that all of it is there
+    if (P.grad_u == nullptr) P.grad_u = dalloc<double>((size_t)P.nt);
+    if (P.grad_part == nullptr) P.grad_part = dalloc<double>((size_t)P.K);
+    std::vector<std::vector<double>> D;   // of the PSD at hand
+    P.grad_H = fold_rows<double>(P, 3, P.npsd, N, [&](int p, int c) {
+        const mm_psd& q = P.h_psd[(size_t)p];
+        if (c == 0) D = toeplitz_row_derivatives(q.sigma, q.fknee, q.alpha, P.L_grid, P.fsamp, P.lambda, P.window);
+        return overlap_save_spectrum(D[(size_t)c], N);
+    });
 }
 
 // dL/dd = N^-1 P mu and dL/dtheta[p][c] = u^T (dN^-1/dtheta_pc) (d - P m), mu = A^-1 g.

@@ -57,14 +57,14 @@ struct ToeplitzDev {
     int cluster = 1;         // CTAs per tile (2 or 4: split across a thread-block cluster)
     int ntiles = 0;
     Tile* tiles = nullptr;   // [ntiles]
-    void* twiddle = nullptr; // T[B/4 + 1]: cos(2 pi k / B) (cluster blocks)
+    void* twiddle = nullptr; // T[B/4 + 1]: cos(2 pi k / B) (FP32: cluster blocks)
     void* ptw = nullptr;     // T2[...]: per-pass twiddles of the N-point FFT (not FP32)
     // FP32 blocks of 2^14 and 2^15 reals (toeplitz_ws.cu): twiddle tables, spectra in the kernel's
     // order, and the plan's input buffers
     void* ws_tab = nullptr;
     void* ws_H = nullptr;
     float* ws_scratch = nullptr;
-    void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N (fold_split_spectra);
+    void* H = nullptr;       // T[npsd][split_size(N)]: kernel spectrum / N (fold_split_spectrum);
                              // FP32: T[npsd][N + 1], divided by another 4 (split_chain)
 };
 
@@ -168,7 +168,7 @@ struct Plan {
     ToeplitzDev tz64, tz32;
     float* ws_scratch = nullptr;   // input buffers of the persistent kernel (toeplitz_ws.cu), or null
     ToeplitzDev tzdf;              // double-float tables (refinement residual)
-    std::vector<std::vector<double>> spec;   // spectra of the rows while tables are built (N = spec_n)
+    std::vector<std::vector<double>> spec;   // spectra of the rows while tables are built (N = spec_n), if few
     int64_t spec_n = 0;
     mutable int64_t tile_count[20] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
 
@@ -254,11 +254,12 @@ bool symbol_positive(const std::vector<double>& t);
 std::vector<std::vector<double>> toeplitz_row_derivatives(double sigma, double fknee, double alpha, int64_t L,
                                                           double fsamp, int lam, int window);
 std::vector<double> overlap_save_spectrum(const std::vector<double>& t, int64_t N);
-// values of a folded spectrum: alpha [N], beta [N/2 + 1], sines [N/2 + 1], the number of chained
-// bins, one of padding
-__host__ __device__ constexpr int64_t split_size(int64_t N) { return 2 * N + 4; }
+// values of a folded spectrum: alpha [N], beta [N/2 + 1], the number of chained bins
+__host__ __device__ constexpr int64_t split_size(int64_t N) { return N + N / 2 + 2; }
 constexpr double SPLIT_RATIO = 0.5;   // of H_k and H_{N-k}: below it a pair of bins is chained
-std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& spectra, int64_t N);
+// cos(2 pi k / B), k = 0..B/4: the quarter wave (sin from the other end)
+std::vector<double> quarter_wave(int64_t B);
+void fold_split_spectrum(const std::vector<double>& h, int64_t N, const std::vector<double>& quarter, double* out);
 // per-pass Stockham twiddles of an N = 2^logn point FFT as interleaved (cos, sin)
 std::vector<double> pass_twiddle_table(int logn);
 double rcond_sym3(const double B[6]);
@@ -290,7 +291,7 @@ void launch_toeplitz_f32_packed(const Plan& P, const float* x, bool pack, float*
                                 cudaStream_t s);
 bool ws_supported(int logn);
 std::vector<float> ws_tables(int logn);
-std::vector<float> ws_spectra(const std::vector<std::vector<double>>& spectra, int logn);
+void ws_append_spectrum(const std::vector<double>& h, int logn, std::vector<float>& out);
 size_t ws_scratch_floats(int num_sms);
 template <typename T>
 size_t toeplitz_smem_bytes(int logn);

@@ -152,49 +152,40 @@ std::vector<double> overlap_save_spectrum(const std::vector<double>& t, int64_t 
     return h;
 }
 
-// Overlap-save spectra h (k = 0..N, over 2N points; overlap_save_spectrum) for the product of a
-// packed real block (toeplitz.cuh, split_product), split_size(N) values per row: alpha [N],
-// beta [N/2 + 1], sine [N/2 + 1], kc.  With W = exp(-i pi k / N) = c - i s,
-// hs = (h_k + h_{N-k}) / 2 and hd = (h_k - h_{N-k}) / 2,
+std::vector<double> quarter_wave(int64_t B) {
+    std::vector<double> c((size_t)(B / 4 + 1));
+    for (int64_t k = 0; k <= B / 4; ++k) c[(size_t)k] = std::cos(2.0 * 3.14159265358979323846 * (double)k / (double)B);
+    return c;
+}
+
+// Overlap-save spectrum h (k = 0..N, over B = 2N points; overlap_save_spectrum) for the product
+// of a packed real block (toeplitz.cuh, split_product), split_size(N) values: alpha [N],
+// beta [N/2 + 1], kc.  With W = exp(-i pi k / N) = c - i s, hs = (h_k + h_{N-k}) / 2 and
+// hd = (h_k - h_{N-k}) / 2,
 //   alpha_k = hs - s hd  (k = 0..N-1),   beta_k = c hd  (k = 0..N/2; beta_{N-k} = beta_k)
 // for the pairs of bins k, N - k whose values are of one size, |h| within a factor 1 /
 // SPLIT_RATIO.  The rounding errors of a folded product are those of the larger value in both
 // bins: the pairs up to the last one with values further apart, k < kc (1/f noise: up to about
 // its knee; a multiple of 32, or all N/2 + 1), go through the chain (split_chain) and hold
-//   alpha_k = h_k / 4, alpha_{N-k} = h_{N-k} / 4 (h_N / 4 in beta_0), beta_k = c, sine_k = s.
-std::vector<double> fold_split_spectra(const std::vector<std::vector<double>>& spectra, int64_t N) {
-    const int64_t hs = split_size(N);
-    std::vector<double> sn((size_t)(N / 2 + 1)), cs((size_t)(N / 2 + 1));   // sin is even about N / 2
-    for (int64_t k = 0; k <= N / 2; ++k) {
-        const double th = 3.14159265358979323846 * (double)k / (double)N;
-        sn[(size_t)k] = std::sin(th);
-        cs[(size_t)k] = std::cos(th);
+//   alpha_k = h_k / 4, alpha_{N-k} = h_{N-k} / 4 (h_N / 4 in beta_0).
+// quarter: quarter_wave(B).
+void fold_split_spectrum(const std::vector<double>& h, int64_t N, const std::vector<double>& quarter, double* out) {
+    double* be = out + N;
+    int64_t kc = N / 2 + 1;
+    while (kc > 0) {
+        const double a = std::fabs(h[(size_t)(kc - 1)]), b = std::fabs(h[(size_t)(N - kc + 1)]);
+        if (!(std::min(a, b) >= SPLIT_RATIO * std::max(a, b))) break;
+        --kc;
     }
-    std::vector<double> f((size_t)((int64_t)spectra.size() * hs), 0.0);
-    for (size_t p = 0; p < spectra.size(); ++p) {
-        const std::vector<double>& h = spectra[p];
-        double* al = f.data() + (int64_t)p * hs;
-        double* be = al + N;
-        double* si = be + N / 2 + 1;
-        int64_t kc = N / 2 + 1;
-        while (kc > 0) {
-            const double a = std::fabs(h[(size_t)(kc - 1)]), b = std::fabs(h[(size_t)(N - kc + 1)]);
-            if (!(std::min(a, b) >= SPLIT_RATIO * std::max(a, b))) break;
-            --kc;
-        }
-        kc = std::min((kc + 31) / 32 * 32, N / 2 + 1);
-        for (int64_t k = 0; k < N; ++k) {
-            const int64_t m = k <= N / 2 ? k : N - k;
-            const double sum = 0.5 * (h[(size_t)k] + h[(size_t)(N - k)]);
-            const double dif = 0.5 * (h[(size_t)k] - h[(size_t)(N - k)]);
-            al[k] = m < kc ? 0.25 * h[(size_t)k] : sum - sn[(size_t)m] * dif;
-            if (k > N / 2) continue;
-            be[k] = m < kc ? (k == 0 ? 0.25 * h[(size_t)N] : cs[(size_t)k]) : cs[(size_t)k] * dif;
-            si[k] = sn[(size_t)k];
-        }
-        si[N / 2 + 1] = (double)kc;
+    kc = std::min((kc + 31) / 32 * 32, N / 2 + 1);
+    for (int64_t k = 0; k < N; ++k) {
+        const int64_t m = k <= N / 2 ? k : N - k;   // the sine is even about N / 2
+        const double sum = 0.5 * (h[(size_t)k] + h[(size_t)(N - k)]);
+        const double dif = 0.5 * (h[(size_t)k] - h[(size_t)(N - k)]);
+        out[k] = m < kc ? 0.25 * h[(size_t)k] : sum - quarter[(size_t)(N / 2 - m)] * dif;
+        if (k <= N / 2) be[k] = m < kc ? (k == 0 ? 0.25 * h[(size_t)N] : 0.0) : quarter[(size_t)k] * dif;
     }
-    return f;
+    be[N / 2 + 1] = (double)kc;
 }
 
 // Twiddles of the in-shared-memory Stockham FFT (toeplitz.cuh): for every pass after the

@@ -67,9 +67,9 @@ __device__ __forceinline__ dfl2 ldc(const dfl2* p) {
 template <typename T>
 struct TzArgs {
     const Tile* tiles;
-    const T* twiddle;      // [N/2 + 1]: cos(2 pi k / B), cross-CTA step of the cluster blocks
+    const T* twiddle;      // [N/2 + 1]: cos(2 pi k / B), cross-CTA step of the cluster blocks, chained bins
     const typename Cx<T>::type* ptw;  // per-pass FFT twiddles (ptw_offset)
-    const T* H;            // [npsd][split_size(N)] (fold_split_spectra); FP32: [npsd][N + 1] spectra / 4
+    const T* H;            // [npsd][split_size(N)] (fold_split_spectrum); FP32: [npsd][N + 1] spectra / 4
     const In<T>* y;        // time-domain input (mode 0)
     const double* yd;      // FP64 time-domain input (modes 2, 4, 5)
     const In<T>* x;        // map (gather modes)
@@ -725,7 +725,7 @@ __device__ __forceinline__ void split_chain(typename Cx<T>::type u1, typename Cx
 }
 
 // split_product: the same written out.  The chain is linear in u1 and conj(u2) with real
-// coefficients that depend on the kernel and k alone (fold_split_spectra):
+// coefficients that depend on the kernel and k alone (fold_split_spectrum):
 //   V_k = alpha_k u1 + i beta_k conj(u2),   V_{N-k} = alpha_{N-k} u2 + i beta_k conj(u1),
 // eight operations for the pair and no twiddle, where the chain takes 44 (one A x in FP64 on
 // 2^22 samples at lambda = 4096: 1.003 -> 0.924 ms, FP64-pipe bound).
@@ -748,27 +748,26 @@ __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename 
     V2.y = -(a2 * u2.y + b * u1.x);
 }
 
-// A row of fold_split_spectra (FP64, double-float): the product of bins k and N - k, k < N, with
-// a1 = alpha_k and a2 = alpha_{N-k} (alpha_0 for k = 0) read ahead by the caller.
+// A row of fold_split_spectrum (FP64, double-float) and the quarter-wave cosine table: the
+// product of bins k and N - k, k < N, with a1 = alpha_k and a2 = alpha_{N-k} (alpha_0 for k = 0)
+// read ahead by the caller.
 template <typename T, int N>
 struct SplitRow {
-    const T *al, *be, *si;
+    const T *al, *be, *quarter;
     int kc;
-    __device__ __forceinline__ explicit SplitRow(const T* row) : al(row), be(row + N), si(row + N + N / 2 + 1) {
-        const T v = si[N / 2 + 1];
+    __device__ __forceinline__ SplitRow(const T* row, const T* q) : al(row), be(row + N), quarter(q) {
+        const T v = be[N / 2 + 1];
         if constexpr (std::is_same<T, double>::value) kc = (int)v;
         else kc = (int)v.hi;
     }
     __device__ __forceinline__ void product(typename Cx<T>::type u1, typename Cx<T>::type u2, int k, T a1, T a2,
                                             typename Cx<T>::type& V1, typename Cx<T>::type& V2) const {
         const int m = k <= N / 2 ? k : N - k;
-        const T b = be[m];
         if (m < kc) {
-            const T sw = si[m];
-            if (k == 0) split_chain<T>(u1, u2, (T)1.0, sw, a1, b, V1, V2);
-            else split_chain<T>(u1, u2, k <= N / 2 ? b : -b, sw, a1, a2, V1, V2);
+            const T c = quarter[m];
+            split_chain<T>(u1, u2, k <= N / 2 ? c : -c, quarter[N / 2 - m], a1, k == 0 ? be[0] : a2, V1, V2);
         } else {
-            split_product<T>(u1, u2, a1, a2, b, V1, V2);
+            split_product<T>(u1, u2, a1, a2, be[m], V1, V2);
         }
     }
 };
@@ -820,7 +819,7 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
         }
         if (tid == 0) product(N / 2, __ldg(H + N / 2), __ldg(H + N / 2));
     } else {
-        const SplitRow<T, N> row(A.H + tile.psd * split_size(N));
+        const SplitRow<T, N> row(A.H + tile.psd * split_size(N), A.twiddle);
         for (int k = tid; k <= N / 2; k += NT) {
             const int k2 = (N - k) & (N - 1);
             C2 V1, V2;
@@ -950,8 +949,10 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     constexpr int64_t HS = F32 ? N + 1 : split_size(N);
     const T* al = A.H + tile.psd * HS;
     // bins k and N - k (FP32: the chain, al = the spectrum itself, h1 and h2 its values)
-    using Row = typename std::conditional<F32, const T*, SplitRow<T, N>>::type;
-    const Row row(al);
+    struct NoRow {
+        __device__ NoRow(const T*, const T*) {}
+    };
+    const typename std::conditional<F32, NoRow, SplitRow<T, N>>::type row(al, A.twiddle);
     auto product = [&](C2 u1, C2 u2, int k, T h1, T h2, C2& V1, C2& V2) {
         if constexpr (F32) {
             float sw, cw;

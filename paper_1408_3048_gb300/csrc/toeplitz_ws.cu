@@ -134,28 +134,25 @@ std::vector<float> ws_tables(int logn) {
 // N - k; then [RM], the first RM / 2 bins of sub-block 1 (task 0) and their partners.
 int64_t ws_spectrum_size(int logn) { return (int64_t)(2 * WS_TASKS + 1) * ((1 << logn) / 4096); }
 
-std::vector<float> ws_spectra(const std::vector<std::vector<double>>& spectra, int logn) {
+void ws_append_spectrum(const std::vector<double>& h, int logn, std::vector<float>& out) {
     const int N = 1 << logn, RM = N / 4096;
-    const int64_t sz = ws_spectrum_size(logn), part = (int64_t)WS_TASKS * RM;
-    std::vector<float> out(spectra.size() * (size_t)sz, 0.f);
-    for (size_t q = 0; q < spectra.size(); ++q) {
-        const std::vector<double>& h = spectra[q];
-        float* o = out.data() + q * (size_t)sz;
-        for (int task = 0; task < WS_TASKS; ++task) {
-            int p, pm;
-            ws_task_host(task, p, pm);
-            const int k0 = brv(p, 12);
-            for (int e = 0; e < RM; ++e) {
-                o[(int64_t)task * RM + e] = (float)(0.25 * h[(size_t)(k0 + 4096 * e)]);
-                o[part + (int64_t)task * RM + e] = (float)(0.25 * h[(size_t)(N - k0 - 4096 * e)]);
-            }
-        }
-        for (int e = 0; e < RM / 2; ++e) {
-            o[2 * part + e] = (float)(0.25 * h[(size_t)(2048 + 4096 * e)]);
-            o[2 * part + RM / 2 + e] = (float)(0.25 * h[(size_t)(N - 2048 - 4096 * e)]);
+    const int64_t part = (int64_t)WS_TASKS * RM;
+    const size_t at = out.size();
+    out.resize(at + (size_t)ws_spectrum_size(logn));
+    float* o = out.data() + at;
+    for (int task = 0; task < WS_TASKS; ++task) {
+        int p, pm;
+        ws_task_host(task, p, pm);
+        const int k0 = brv(p, 12);
+        for (int e = 0; e < RM; ++e) {
+            o[(int64_t)task * RM + e] = (float)(0.25 * h[(size_t)(k0 + 4096 * e)]);
+            o[part + (int64_t)task * RM + e] = (float)(0.25 * h[(size_t)(N - k0 - 4096 * e)]);
         }
     }
-    return out;
+    for (int e = 0; e < RM / 2; ++e) {
+        o[2 * part + e] = (float)(0.25 * h[(size_t)(2048 + 4096 * e)]);
+        o[2 * part + RM / 2 + e] = (float)(0.25 * h[(size_t)(N - 2048 - 4096 * e)]);
+    }
 }
 
 // ---------------------------------------------------------------------- butterflies

@@ -6,6 +6,7 @@ import ctypes
 import os
 import shutil
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -25,6 +26,10 @@ def lib(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("fake") / "libfake.so")
     subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-I", inc, "-o", so,
                     os.path.join(HERE, "fake_cuda.cpp"), *objs, "-lpthread"], check=True)
+    return load(so)
+
+
+def load(so):
     L = ctypes.CDLL(so)
     for name, (res, args) in mm._SIGS.items():
         fn = getattr(L, name)
@@ -153,3 +158,26 @@ def test_one_set_of_input_buffers_per_plan(lib):
         held.append(lib.fake_live_bytes() - before)
         p.close()
     assert buffers < held[0] < held[1] + buffers // 8
+
+
+MANY_PSDS = r"""
+import resource, sys
+sys.path[:0] = [{here!r}, {root!r}]
+import test_host_alloc as t
+L = t.load({so!r})
+rss = lambda: 1024 * resource.getrusage(resource.RUSAGE_SELF).ru_maxrss
+small = t.Plan(L, [20000], 1000, 1, npsd=2, fft_log2_f64=14, fft_log2_f32=14)
+small.close()
+base, dev = rss(), L.fake_live_bytes()
+p = t.Plan(L, [20000], 1000, 1, npsd=1500, fft_log2_f64=14, fft_log2_f32=14)
+print(rss() - base - (L.fake_peak_bytes(0) - dev))
+"""
+
+
+def test_spectra_of_many_psds_one_at_a_time(lib):
+    """Building a plan of many PSDs holds one arithmetic's table on the host beside the device's
+    (147 MB of folded spectra here), not the spectra of all rows in several copies."""
+    code = MANY_PSDS.format(here=HERE, root=os.path.dirname(HERE), so=lib._name)
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, check=True).stdout
+    table = 1500 * (8192 + 4096 + 2) * 8
+    assert int(out) < 1.5 * table, (int(out), table)

@@ -1,4 +1,4 @@
-"""Spectra of the FP64 and double-float block product (fold_split_spectra in csrc/plan_host.cpp)
+"""Spectra of the FP64 and double-float block product (fold_split_spectrum in csrc/plan_host.cpp)
 on the CPU: the product that the kernels form from a row, folded pairs of bins and chained
 ones, equals the circular convolution with the row's spectrum; which bins are chained."""
 import os
@@ -20,9 +20,10 @@ int main() {
     if (std::scanf("%lld", &N) != 1) return 2;
     std::vector<double> h((size_t)N + 1);
     for (auto& x : h) if (std::scanf("%lf", &x) != 1) return 2;
-    const std::vector<double> f = mm::fold_split_spectra({h, h}, N);
-    if ((long long)f.size() != 2 * mm::split_size(N)) return 3;
+    std::vector<double> f((size_t)mm::split_size(N)), q = mm::quarter_wave(2 * N);
+    mm::fold_split_spectrum(h, N, q, f.data());
     for (double x : f) std::printf("%.17g\n", x);
+    for (double x : q) std::printf("%.17g\n", x);
     return 0;
 }
 """
@@ -41,20 +42,21 @@ def fold(tmp_path_factory):
         text = f"{len(h) - 1}\n" + "\n".join(repr(float(v)) for v in h)
         out = subprocess.run([str(d / "driver")], input=text, capture_output=True, text=True, check=True).stdout
         f = np.array([float(v) for v in out.split()])
-        assert np.array_equal(f[:f.size // 2], f[f.size // 2:])   # the two rows
-        return f[:f.size // 2]
+        N = len(h) - 1
+        assert f.size == N + N // 2 + 2 + N // 2 + 1
+        return f[:-(N // 2 + 1)], f[-(N // 2 + 1):]
     return run
 
 
-def _product(f, U, N):
+def _product(f, quarter, U, N):
     """V from U as SplitRow::product forms it, bins k and N - k together."""
-    al, be, si, kc = f[:N], f[N:N + N // 2 + 1], f[N + N // 2 + 1:N + 2 * (N // 2 + 1)], int(f[2 * N + 2])
+    al, be, kc = f[:N], f[N:N + N // 2 + 1], int(f[-1])
     V = np.empty(N, complex)
     for k in range(N // 2 + 1):
         u1, u2 = U[k], U[-k % N]
         if k < kc:
-            c, h2 = (1.0, be[0]) if k == 0 else (be[k], al[N - k])
-            W = c - 1j * si[k]
+            h2 = be[0] if k == 0 else al[N - k]
+            W = quarter[k] - 1j * quarter[N // 2 - k]
             E, O = u1 + np.conj(u2), -1j * (u1 - np.conj(u2))
             Z1, Z2 = al[k] * (E + W * O), h2 * (E - W * O)
             S, D = Z1 + Z2, np.conj(W) * (Z1 - Z2)
@@ -77,9 +79,9 @@ def _spectra(N):
 @pytest.mark.parametrize("kind", ["white", "knee", "zero", "falling", "signs", "rough", "steep"])
 def test_product(fold, kind, N):
     h = _spectra(N)[kind]
-    f = fold(h)
+    f, quarter = fold(h)
     y = np.random.default_rng(1).standard_normal(2 * N)
-    V, kc = _product(f, np.fft.fft(y[0::2] + 1j * y[1::2]), N)
+    V, kc = _product(f, quarter, np.fft.fft(y[0::2] + 1j * y[1::2]), N)
     v = np.fft.ifft(V)
     z = np.stack([v.real, v.imag], 1).ravel()
     ref = np.fft.irfft(np.fft.rfft(y) * h, n=2 * N)
