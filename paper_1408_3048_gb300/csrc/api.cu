@@ -298,25 +298,27 @@ static double block_us(const Plan& P, int logn, int64_t tiles) {
 // one sequence, which saves the partly filled last tile of every interval but one.  A run
 // is packed only when that gives fewer tiles and no tile needs more than TILE_SEGS
 // segments; otherwise each interval is tiled on its own (one segment per tile).
-// Outputs of a full tile: B - 2 lambda, rounded down to a multiple of 4 where that leaves any
-// (the distance of two windows is then one that the FP32 kernel copies between them).
-static int64_t tile_outputs(int64_t B, int64_t lam) {
-    const int64_t v = B - 2 * lam;
-    return v >= 4 ? v & ~int64_t(3) : v;
-}
-static std::vector<Tile> make_tiles(const Plan& P, int64_t B) {
+//
+// ws: tiles of the persistent FP32 kernel.  It copies the positions that two windows share
+// from one to the next where their distance is a multiple of four, and stores four outputs as
+// one 16-byte word where the shift from position to time is one.  Its runs therefore take
+// B - 2 lambda rounded down to a multiple of four (where that leaves any) as the outputs of a
+// full tile, and up to three more zeros ahead of an interval.  Without: I/Q/U, 2^24 samples,
+// lambda = 4095 157 us instead of 123; T, 2^26 samples, lambda = 1023 400 instead of 291; N^-1
+// on 8e6 samples, lambda = 2048 99 instead of 79.  So a run is laid out that way unless it
+// then needs over a fifth more tiles (intervals just as long as the outputs of a tile; a band
+// two or three samples short of half a block).  The other kernels gain nothing from it.
+static std::vector<Tile> make_tiles(const Plan& P, int64_t B, bool ws) {
     const int64_t lam = P.lambda;
-    const int64_t Lv = tile_outputs(B, lam);
     std::vector<Tile> out;
-    auto tile_run = [&](int i0, int i1, std::vector<Tile>& dst) -> bool {
+    auto tile_run = [&](int i0, int i1, bool fours, std::vector<Tile>& dst) -> bool {
+        const int64_t v = B - 2 * lam, Lv = fours && v >= 4 ? v & ~int64_t(3) : v;
         // virtual start of each interval of the run [i0, i1)
         std::vector<int64_t> V((size_t)(i1 - i0));
         int64_t vlen = 0;
         for (int i = i0; i < i1; ++i) {
             if (i > i0) vlen += lam;
-            // up to three more zeros, so that the shift from position to time is a multiple of
-            // four: the FP32 kernel then stores four outputs as one 16-byte word
-            vlen += (P.h_ioff[i] - lam - vlen) & 3;
+            if (fours) vlen += (P.h_ioff[i] - lam - vlen) & 3;
             V[(size_t)(i - i0)] = vlen;
             vlen += P.h_ioff[i + 1] - P.h_ioff[i];
         }
@@ -349,24 +351,35 @@ static std::vector<Tile> make_tiles(const Plan& P, int64_t B) {
         }
         return true;
     };
+    auto lay_out = [&](int i0, int i1, bool fours) {
+        std::vector<Tile> single, packed;
+        for (int i = i0; i < i1; ++i) tile_run(i, i + 1, fours, single);
+        const bool pack = i1 - i0 > 1 && tile_run(i0, i1, fours, packed) && packed.size() < single.size();
+        return pack ? packed : single;
+    };
     for (int i0 = 0; i0 < P.K;) {
         int i1 = i0 + 1;
         while (i1 < P.K && P.h_ipsd[i1] == P.h_ipsd[i0]) ++i1;
-        std::vector<Tile> single, packed;
-        for (int i = i0; i < i1; ++i) tile_run(i, i + 1, single);
-        if (i1 - i0 > 1 && tile_run(i0, i1, packed) && packed.size() < single.size())
-            out.insert(out.end(), packed.begin(), packed.end());
-        else
-            out.insert(out.end(), single.begin(), single.end());
+        std::vector<Tile> run = lay_out(i0, i1, false);
+        if (ws) {
+            std::vector<Tile> fours = lay_out(i0, i1, true);
+            if (5 * fours.size() <= 6 * run.size()) run.swap(fours);
+        }
+        out.insert(out.end(), run.begin(), run.end());
         i0 = i1;
     }
     return out;
 }
 
+// Whether FP32 blocks of 2^logn packed points run on the persistent kernel.
+template <typename T>
+static bool ws_block(int logn) { return sizeof(T) == 4 && ws_supported(logn); }
+
 // Number of tiles of a block, kept per plan while it is built (three arithmetics ask).
+template <typename T>
 static int64_t overlap_tiles(const Plan& P, int logn) {
-    int64_t& n = P.tile_count[logn];
-    if (n < 0) n = (int64_t)make_tiles(P, int64_t(2) << logn).size();
+    int64_t& n = P.tile_count[ws_block<T>(logn)][logn];
+    if (n < 0) n = (int64_t)make_tiles(P, int64_t(2) << logn, ws_block<T>(logn)).size();
     return n;
 }
 
@@ -388,7 +401,7 @@ static std::vector<std::pair<double, int>> block_candidates(const Plan& P, int R
         const int64_t N = int64_t(1) << logn;
         const int64_t Lv = 2 * N - 2 * (int64_t)P.lambda;
         if (Lv < 1) continue;
-        c.push_back({block_us<T>(P, logn, overlap_tiles(P, logn) * R), logn});
+        c.push_back({block_us<T>(P, logn, overlap_tiles<T>(P, logn) * R), logn});
     }
     std::stable_sort(c.begin(), c.end());
     return c;
@@ -455,7 +468,7 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
     tz.logn = choose_logn<T>(P, forced_log2B, &tz.cluster);
     const int64_t N = int64_t(1) << tz.logn;
     const int64_t B = 2 * N;
-    const std::vector<Tile> tiles = make_tiles(P, B);
+    const std::vector<Tile> tiles = make_tiles(P, B, ws_block<T>(tz.logn));
     tz.ntiles = (int)tiles.size();
     tz.tiles = dalloc<Tile>(tiles.size());
     h2d(tz.tiles, tiles.data(), tiles.size() * sizeof(Tile), P.stream);
@@ -478,7 +491,7 @@ static void build_toeplitz(Plan& P, ToeplitzDev& tz, int forced_log2B) {
     auto spectrum = [&](int p, int) { return plan_spectrum(P, p, N); };
     if constexpr (sizeof(T) == 4) {
         std::vector<float> H;
-        if (tz.cluster == 1 && ws_supported(tz.logn)) {
+        if (ws_block<T>(tz.logn)) {
             const std::vector<float> tab = ws_tables(tz.logn);
             tz.ws_tab = dalloc<float>(tab.size());
             h2d(tz.ws_tab, tab.data(), tab.size() * 4, P.stream);
@@ -511,7 +524,7 @@ static void build_toeplitz_df(Plan& P, int forced_log2B) {
     const int64_t N = int64_t(1) << tz.logn;
     const int64_t B = 2 * N;
     try {
-        const std::vector<Tile> tiles = make_tiles(P, B);
+        const std::vector<Tile> tiles = make_tiles(P, B, false);
         tz.ntiles = (int)tiles.size();
         tz.tiles = dalloc<Tile>(tiles.size());
         h2d(tz.tiles, tiles.data(), tiles.size() * sizeof(Tile), P.stream);
@@ -2005,7 +2018,7 @@ static void ensure_batch_tables(PlanHolder& P, int R, int want = -1) {
     double real_cost = -1.0;
     if (P.tz32.logn != 0) {
         const int logn = batch_real_logn(P, BATCH_RMAX);
-        real_cost = block_us<float>(P, logn, overlap_tiles(P, logn) * BATCH_RMAX);
+        real_cost = block_us<float>(P, logn, overlap_tiles<float>(P, logn) * BATCH_RMAX);
     }
     if (best < 0 && real_cost < 0.0) throw Error{MM_ERR_ARG, "lambda too large for the batched FFT blocks"};
     if ((want == BATCH_PAIR && best < 0) || (want == BATCH_REAL && real_cost < 0.0))

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <array>
 #include <string>
 #include <utility>
 #include <vector>
@@ -36,7 +37,8 @@ struct Tile {
     int32_t pe[TILE_SEGS];
     int32_t nout;
     int32_t psd;
-    int32_t cont;   // positions from the window of the tile before, of the same run, to this one's (0: none)
+    int32_t cont;   // positions from the window of the tile before, of the same run, to this one's, a
+                    // multiple of 4 (0: none)
     int32_t unused;
 };
 
@@ -170,7 +172,10 @@ struct Plan {
     ToeplitzDev tzdf;              // double-float tables (refinement residual)
     std::vector<std::vector<double>> spec;   // spectra of the rows while tables are built (N = spec_n), if few
     int64_t spec_n = 0;
-    mutable int64_t tile_count[20] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
+    mutable std::array<std::array<int64_t, 20>, 2> tile_count;   // by layout and logn, -1: not counted yet
+    Plan() {
+        for (auto& c : tile_count) c.fill(-1);
+    }
 
     // block-Jacobi: inverse blocks, symmetric packed (a00 a01 a02 a11 a12 a22) or 1
     double* bd64 = nullptr;        // [npix_obs][ncomp == 3 ? 6 : 1]

@@ -181,3 +181,22 @@ def test_spectra_of_many_psds_one_at_a_time(lib):
     out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, check=True).stdout
     table = 1500 * (8192 + 4096 + 2) * 8
     assert int(out) < 1.5 * table, (int(out), table)
+
+
+# (lambda, log2 block of FP64 and FP32, interval length): as long as a tile's outputs, which are
+# no multiple of four, or a band that leaves six outputs
+@pytest.mark.parametrize("lam,logs,length,tiles", [(1001, (12, 12), 2094, 1), (512, (12, 12), 3071, 1), (1001, (14, 14), 14382, 1),
+                                                   (2001, (15, 15), 28766, 1), (8189, (14, 14), 12000, 2000)])
+def test_interval_of_a_tiles_outputs_takes_one_tile(lib, lam, logs, length, tiles):
+    p = Plan(lib, [length] * 3, lam, 1, fft_log2_f64=logs[0], fft_log2_f32=logs[1])
+    v = np.zeros(p.nt)
+    want = tiles * 6
+    for prec, cl in ((mm.MM_FP64, {15: 2}.get(logs[0], 1)), (mm.MM_FP32, 1)):
+        lib.fake_clear_launches()
+        assert lib.mm_apply_ninv(p.h, prec, v.ctypes.data, v.ctypes.data) == mm.MM_OK
+        (name, grid, _), = launches(lib)
+        if "toeplitz_ws" in name:   # CTAs of several tiles each
+            assert grid == -(-want // -(-want // (152 << (15 - logs[1]))))
+        else:
+            assert grid == want * cl, name
+    p.close()
