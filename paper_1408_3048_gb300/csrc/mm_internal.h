@@ -322,7 +322,6 @@ void launch_scatter_sliced(const Plan& P, const T* z, T* w, const T* p, double* 
                            const int* done, cudaStream_t s);
 template <typename T>
 void launch_batch_scatter_sliced(const Plan& P, const T* Z, T* W, int R, const int* done, cudaStream_t s);
-int sliced_blocks(const Plan& P, int wpb, int S);
 void launch_bd_build(const Plan& P, double* bd64, float* bd32, cudaStream_t s);
 // merged a priori coarse space Z_S (Sec. 3.3.1), r groups of consecutive intervals, into
 // Z [r][n] FP64 (zeroed here)
