@@ -258,13 +258,16 @@ __global__ void __launch_bounds__(WPB * 32, (sl_min_blocks<T, NC, WPB>())) slice
 }
 
 // Warps per slice: enough of them for half the chip's warps, each with at least a batch of
-// steps; groups: walks over every slice (groups of right-hand sides).  (More parts shorten the
-// last, partly filled wave of blocks but also the slices' runs: four warps per slice on 8192
-// slices of 64 steps took 51 us, one 47.)
-static int sliced_parts(const Plan& P, int groups) {
+// steps.  (More parts shorten the last, partly filled wave of blocks but also the slices' runs:
+// four warps per slice on 8192 slices of 64 steps took 51 us, one 47.)  groups: of right-hand
+// sides, each a walk over every slice; a batch's warps have several loads in flight for a step
+// and fill the chip four times as early (512 slices of 64 steps, four groups of four columns:
+// one warp per slice, with two a batched solve took 2 % longer).
+static int sliced_parts(const Plan& P, int groups = 0) {
     const int64_t steps = P.sl_count > 0 ? P.sl_steps / P.sl_count : 0;
+    const int64_t enough = (int64_t)P.num_sms * (groups > 0 ? 8 : 32), walks = (int64_t)P.sl_count * std::max(groups, 1);
     int S = 1;
-    while (S < 32 && (int64_t)P.sl_count * groups * S < (int64_t)P.num_sms * 32 && steps / (2 * S) >= SL_U) S *= 2;
+    while (S < 32 && walks * S < enough && steps / (2 * S) >= SL_U) S *= 2;
     return S;
 }
 
@@ -279,7 +282,7 @@ static int sliced_blocks(const Plan& P, int wpb, int S) {
 template <typename T, int NC, bool DOT, bool ANG>
 static void sliced_launch(const Plan& P, const typename W2<T>::type* sw, const float* sang, const T* z, T* w,
                           const int* done, SlicedDot sd, cudaStream_t s) {
-    const int S = sliced_parts(P, 1);
+    const int S = sliced_parts(P);
     const int32_t* so = P.sl_off;
     const int32_t* st = P.sl_t;
     if (S <= 8)
@@ -322,132 +325,154 @@ template void launch_scatter_sliced<float>(const Plan&, const float*, float*, co
 
 // ------------------------------------------------------------- many right-hand sides
 // The same walk for RC right-hand sides at a time (grid.y; four in FP32, two in FP64): a step's
-// indices and weights are read once for them.  PARTS: S warps per slice as above, where few pixels
-// and few columns have too few slices for the chip (T, 64 pixels of 8192 samples, two columns:
-// 505 -> 67 us for A x, the 32-lane form 103); without, S = 1 (the division and the barriers of
-// the other cost 5 % of a 64-column product).
+// indices and weights are read once for them.
 constexpr int SL_BU = 4;
 
-template <typename T, int NC, int RC, int WPB, bool PARTS>
-__global__ void __launch_bounds__(WPB * 32) sliced_batch_kernel(const int32_t* __restrict__ sl_off,
-                                                                const int32_t* __restrict__ st,
-                                                                const typename W2<T>::type* __restrict__ sw,
-                                                                const T* __restrict__ Z, T* __restrict__ W, int nslices,
-                                                                int npix, int64_t nt, int64_t n, int R, int S,
-                                                                const int* done) {
+// a += steps [j, j1) of a slice; z0: the first right-hand side of the group
+template <typename T, int NC, int RC>
+__device__ __forceinline__ void batch_walk(Acc<T> (&a)[RC][NC], int j, int j1, const int32_t* __restrict__ st,
+                                           const typename W2<T>::type* __restrict__ sw, const T* __restrict__ z0, int r0,
+                                           int64_t nt, int R, int lane) {
     using V2 = typename W2<T>::type;
-    if (done != nullptr && *(volatile const int*)done) return;
-    __shared__ T comb[PARTS ? WPB : 1][SL_PIX][RC][2 * NC];   // parts 1 .. S - 1 of their slices
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    const int part = PARTS ? wi % S : 0, grp = PARTS ? wi / S : wi, G = PARTS ? WPB / S : WPB;
-    const int r0 = blockIdx.y * RC;
-    const T* z0 = Z + (size_t)r0 * nt;
-    for (int sb = blockIdx.x * G; sb < nslices; sb += gridDim.x * G) {   // uniform over the block
-        const int s = sb + grp;
-        if (!PARTS && s >= nslices) break;
-        Acc<T> a[RC][NC];
-        int j0 = 0, j1 = 0;
-        if (!PARTS || s < nslices) {
-            j0 = sl_off[s];
-            j1 = sl_off[s + 1];
+    for (; j < j1; j += SL_BU) {
+        int t[SL_BU];
+        V2 ww[SL_BU];
+#pragma unroll
+        for (int u = 0; u < SL_BU; ++u) {
+            const int64_t e = (int64_t)min(j + u, j1 - 1) * 32 + lane;
+            t[u] = j + u < j1 ? __ldg(st + e) : -1;
+            if constexpr (NC == 3) ww[u] = __ldg(sw + e);
         }
-        if constexpr (PARTS) {
-            const int per = (j1 - j0 + S - 1) / S;
-            j0 = min(j1, j0 + part * per);
-            j1 = min(j1, j0 + per);
+        T v[RC][SL_BU];
+#pragma unroll
+        for (int r = 0; r < RC; ++r) {
+            const T* z = z0 + (r0 + r < R ? (size_t)r * nt : 0);
+#pragma unroll
+            for (int u = 0; u < SL_BU; ++u) v[r][u] = z[max(t[u], 0)];
         }
-        for (int j = j0; j < j1; j += SL_BU) {
-            int t[SL_BU];
-            V2 ww[SL_BU];
+#pragma unroll
+        for (int r = 0; r < RC; ++r) {
+            T b[NC] = {};
 #pragma unroll
             for (int u = 0; u < SL_BU; ++u) {
-                const int64_t e = (int64_t)min(j + u, j1 - 1) * 32 + lane;
-                t[u] = j + u < j1 ? __ldg(st + e) : -1;
-                if constexpr (NC == 3) ww[u] = __ldg(sw + e);
-            }
-            T v[RC][SL_BU];
-#pragma unroll
-            for (int r = 0; r < RC; ++r) {
-                const T* z = z0 + (r0 + r < R ? (size_t)r * nt : 0);
-#pragma unroll
-                for (int u = 0; u < SL_BU; ++u) v[r][u] = z[max(t[u], 0)];
-            }
-#pragma unroll
-            for (int r = 0; r < RC; ++r) {
-                T b[NC] = {};
-#pragma unroll
-                for (int u = 0; u < SL_BU; ++u) {
-                    const T x = t[u] >= 0 ? v[r][u] : (T)0;
-                    b[0] += x;
-                    if constexpr (NC == 3) {
-                        b[1] += ww[u].x * x;
-                        b[2] += ww[u].y * x;
-                    }
+                const T x = t[u] >= 0 ? v[r][u] : (T)0;
+                b[0] += x;
+                if constexpr (NC == 3) {
+                    b[1] += ww[u].x * x;
+                    b[2] += ww[u].y * x;
                 }
-#pragma unroll
-                for (int c = 0; c < NC; ++c) a[r][c].add(b[c]);
             }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) a[r][c].add(b[c]);
         }
+    }
+}
+
+template <typename T, int NC, int RC>
+__global__ void __launch_bounds__(256) sliced_batch_kernel(const int32_t* __restrict__ sl_off,
+                                                           const int32_t* __restrict__ st,
+                                                           const typename W2<T>::type* __restrict__ sw,
+                                                           const T* __restrict__ Z, T* __restrict__ W, int nslices,
+                                                           int npix, int64_t nt, int64_t n, int R, const int* done) {
+    if (done != nullptr && *(volatile const int*)done) return;
+    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    const int r0 = blockIdx.y * RC;
+    const T* z0 = Z + (size_t)r0 * nt;
+    for (int s = blockIdx.x * warps + (threadIdx.x >> 5); s < nslices; s += gridDim.x * warps) {
+        Acc<T> a[RC][NC];
+        const int j1 = sl_off[s + 1];
+        batch_walk<T, NC, RC>(a, sl_off[s], j1, st, sw, z0, r0, nt, R, lane);
+        const int q = s * SL_PIX + (lane >> 2);
 #pragma unroll
         for (int r = 0; r < RC; ++r)
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 a[r][c].lanes(1);
                 a[r][c].lanes(2);
+                if ((lane & 3) == 0 && q < npix && r0 + r < R) W[(size_t)(r0 + r) * n + (int64_t)q * NC + c] = a[r][c].total();
             }
-        const int px = lane >> 2, q = s * SL_PIX + px;
-        if constexpr (PARTS) {
-            if ((lane & 3) == 0 && part > 0) {
-#pragma unroll
-                for (int r = 0; r < RC; ++r)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        comb[wi][px][r][2 * c] = a[r][c].hi;
-                        comb[wi][px][r][2 * c + 1] = a[r][c].lo;
-                    }
-            }
-            __syncthreads();
-            if ((lane & 3) == 0 && part == 0)
-                for (int p = 1; p < S; ++p)
-#pragma unroll
-                    for (int r = 0; r < RC; ++r)
-#pragma unroll
-                        for (int c = 0; c < NC; ++c)
-                            a[r][c].merge(comb[wi + p][px][r][2 * c], comb[wi + p][px][r][2 * c + 1]);
-            __syncthreads();
-        }
-        if ((lane & 3) == 0 && part == 0 && q < npix) {
-#pragma unroll
-            for (int r = 0; r < RC; ++r)
-#pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (r0 + r < R) W[(size_t)(r0 + r) * n + (int64_t)q * NC + c] = a[r][c].total();
-        }
     }
 }
 
-template <typename T, int WPB, bool PARTS>
-static void sliced_batch_launch(const Plan& P, const T* Z, T* W, int R, int S, const int* done, cudaStream_t s) {
+// S warps per slice as above, where few pixels and few columns have too few slices for the chip
+// (T, 64 pixels of 8192 samples, two columns: A x 505 -> 67 us, with the 32-lane form 103).  With
+// S = 1 it took 346 us where the kernel above takes 319 (64 columns, 2^22 I/Q/U samples).
+template <typename T, int NC, int RC, int WPB>
+__global__ void __launch_bounds__(WPB * 32) sliced_batch_parts_kernel(const int32_t* __restrict__ sl_off,
+                                                                      const int32_t* __restrict__ st,
+                                                                      const typename W2<T>::type* __restrict__ sw,
+                                                                      const T* __restrict__ Z, T* __restrict__ W,
+                                                                      int nslices, int npix, int64_t nt, int64_t n, int R,
+                                                                      int S, const int* done) {
+    if (done != nullptr && *(volatile const int*)done) return;
+    __shared__ T comb[WPB][SL_PIX][RC][2 * NC];   // parts 1 .. S - 1 of their slices
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int part = wi % S, G = WPB / S;
+    const int r0 = blockIdx.y * RC;
+    const T* z0 = Z + (size_t)r0 * nt;
+    for (int sb = blockIdx.x * G; sb < nslices; sb += gridDim.x * G) {   // uniform over the block
+        const int s = sb + wi / S;
+        Acc<T> a[RC][NC];
+        if (s < nslices) {
+            const int o0 = sl_off[s], o1 = sl_off[s + 1], per = (o1 - o0 + S - 1) / S;
+            const int j0 = min(o1, o0 + part * per);
+            batch_walk<T, NC, RC>(a, j0, min(o1, j0 + per), st, sw, z0, r0, nt, R, lane);
+        }
+        const int px = lane >> 2, q = s * SL_PIX + px;
+#pragma unroll
+        for (int r = 0; r < RC; ++r)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                a[r][c].lanes(1);
+                a[r][c].lanes(2);
+                if ((lane & 3) == 0 && part > 0) {
+                    comb[wi][px][r][2 * c] = a[r][c].hi;
+                    comb[wi][px][r][2 * c + 1] = a[r][c].lo;
+                }
+            }
+        __syncthreads();
+        if ((lane & 3) == 0 && part == 0 && s < nslices && q < npix)
+#pragma unroll
+            for (int r = 0; r < RC; ++r)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    for (int p = 1; p < S; ++p) a[r][c].merge(comb[wi + p][px][r][2 * c], comb[wi + p][px][r][2 * c + 1]);
+                    if (r0 + r < R) W[(size_t)(r0 + r) * n + (int64_t)q * NC + c] = a[r][c].total();
+                }
+        __syncthreads();
+    }
+}
+
+template <typename T, int WPB>
+static void sliced_batch_parts(const Plan& P, const typename W2<T>::type* sw, const T* Z, T* W, int R, int S,
+                               const int* done, cudaStream_t s) {
     constexpr int RC = sizeof(T) == 4 ? 4 : 2;
     const int G = WPB / S;
     const int gx = std::max(1, std::min((P.sl_count + G - 1) / G, P.num_sms * 8));
     const dim3 grid((unsigned)gx, (unsigned)((R + RC - 1) / RC));
-    const typename W2<T>::type* sw = nullptr;
-    if constexpr (sizeof(T) == 4) sw = P.sl_w32;
-    else sw = P.sl_w64;
-    auto kern = P.ncomp == 1 ? sliced_batch_kernel<T, 1, RC, WPB, PARTS> : sliced_batch_kernel<T, 3, RC, WPB, PARTS>;
+    auto kern = P.ncomp == 1 ? sliced_batch_parts_kernel<T, 1, RC, WPB> : sliced_batch_parts_kernel<T, 3, RC, WPB>;
     kern<<<grid, WPB * 32, 0, s>>>(P.sl_off, P.sl_t, sw, Z, W, P.sl_count, P.npix_obs, P.nt, P.n, R, S, done);
-    check_cuda(cudaGetLastError(), "batch scatter launch");
-    note_launch();
 }
 
 template <typename T>
 void launch_batch_scatter_sliced(const Plan& P, const T* Z, T* W, int R, const int* done, cudaStream_t s) {
     constexpr int RC = sizeof(T) == 4 ? 4 : 2;
+    const typename W2<T>::type* sw = nullptr;
+    if constexpr (sizeof(T) == 4) sw = P.sl_w32;
+    else sw = P.sl_w64;
     const int S = sliced_parts(P, (R + RC - 1) / RC);
-    if (S == 1) sliced_batch_launch<T, 8, false>(P, Z, W, R, 1, done, s);
-    else if (S <= 8) sliced_batch_launch<T, 8, true>(P, Z, W, R, S, done, s);
-    else sliced_batch_launch<T, 32, true>(P, Z, W, R, S, done, s);
+    if (S == 1) {
+        const int gx = std::max(1, std::min((P.sl_count + 7) / 8, P.num_sms * 8));
+        const dim3 grid((unsigned)gx, (unsigned)((R + RC - 1) / RC));
+        auto kern = P.ncomp == 1 ? sliced_batch_kernel<T, 1, RC> : sliced_batch_kernel<T, 3, RC>;
+        kern<<<grid, 256, 0, s>>>(P.sl_off, P.sl_t, sw, Z, W, P.sl_count, P.npix_obs, P.nt, P.n, R, done);
+    } else if (S <= 8) {
+        sliced_batch_parts<T, 8>(P, sw, Z, W, R, S, done, s);
+    } else {
+        sliced_batch_parts<T, 32>(P, sw, Z, W, R, S, done, s);
+    }
+    check_cuda(cudaGetLastError(), "batch scatter launch");
+    note_launch();
 }
 template void launch_batch_scatter_sliced<float>(const Plan&, const float*, float*, int, const int*, cudaStream_t);
 template void launch_batch_scatter_sliced<double>(const Plan&, const double*, double*, int, const int*, cudaStream_t);
