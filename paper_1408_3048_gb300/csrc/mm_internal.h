@@ -261,7 +261,7 @@ std::vector<std::vector<double>> toeplitz_row_derivatives(double sigma, double f
 std::vector<double> overlap_save_spectrum(const std::vector<double>& t, int64_t N);
 // values of a folded spectrum: alpha [N], beta [N/2 + 1], the number of chained bins
 __host__ __device__ constexpr int64_t split_size(int64_t N) { return N + N / 2 + 2; }
-constexpr double SPLIT_RATIO = 0.5;   // of H_k and H_{N-k}: below it a pair of bins is chained
+constexpr double SPLIT_RATIO = 0.25;   // of H_k and H_{N-k}: below it a pair of bins is chained
 // cos(2 pi k / B), k = 0..B/4: the quarter wave (sin from the other end)
 std::vector<double> quarter_wave(int64_t B);
 void fold_split_spectrum(const std::vector<double>& h, int64_t N, const std::vector<double>& quarter, double* out);

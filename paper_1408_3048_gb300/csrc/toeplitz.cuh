@@ -737,7 +737,7 @@ __device__ __forceinline__ void split_chain(typename Cx<T>::type u1, typename Cx
 // f_knee = 1 to 2 Hz the FP64 product left 3e-15 to 1e-12 of the lowest modes as rounding, the
 // chain less than 2e-15.  So FP32 takes the chain throughout, FP64 and double-float for the
 // bins where H_k and H_{N-k} differ by more than a factor 1 / SPLIT_RATIO (f_knee = 2 Hz at 100
-// Hz: 1 bin in 12; A x of 2^22 I/Q/U samples 808 -> 813 us, the double-float residual
+// Hz: 1 bin in 20; A x of 2^22 I/Q/U samples 808 -> 813 us, the double-float residual
 // unchanged at 481).
 template <typename T>
 __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename Cx<T>::type u2, T a1, T a2, T b,

@@ -71,7 +71,7 @@ def _spectra(N):
     f = np.arange(N + 1) / N
     rng = np.random.default_rng(3)
     return {"white": np.ones(N + 1), "knee": 1 / (1 + (0.04 / np.maximum(f, 1e-3))**2), "zero": np.zeros(N + 1),
-            "falling": 1 / (1e-3 + f), "signs": np.cos(9 * f), "rough": rng.uniform(0.9, 1.0, N + 1) * (1 + 3 * (f > 0.7)),
+            "falling": 1 / (1e-3 + f), "signs": np.cos(9 * f), "rough": rng.uniform(0.9, 1.0, N + 1) * (1 + 5 * (f > 0.7)),
             "steep": np.maximum(f, 1e-4)**2}
 
 
@@ -86,10 +86,10 @@ def test_product(fold, kind, N):
     z = np.stack([v.real, v.imag], 1).ravel()
     ref = np.fft.irfft(np.fft.rfft(y) * h, n=2 * N)
     assert np.linalg.norm(z - ref) <= 1e-14 * max(np.abs(h).max(), 1e-300) * np.linalg.norm(y)
-    # chained: up to the last pair whose values differ by more than a factor 2, in whole warps
+    # chained: up to the last pair whose values differ by more than a factor 4, in whole warps
     k = np.arange(N // 2 + 1)
     a, b = np.abs(h[k]), np.abs(h[N - k])
-    far = np.flatnonzero(np.minimum(a, b) < 0.5 * np.maximum(a, b))
+    far = np.flatnonzero(np.minimum(a, b) < 0.25 * np.maximum(a, b))
     want = 0 if far.size == 0 else far[-1] + 1
     assert kc == min(-(-want // 32) * 32, N // 2 + 1)
     assert (kc > 0) == (kind not in ("white", "zero"))
