@@ -145,12 +145,21 @@ mm_status mm_autotune_read(mm_plan_t plan, float* ms_f64, float* ms_f32);
  * sorted samples (32, 16 or 8: one, two or four pixels per warp).  32 unless the plan
  * autotunes (opts.autotune), which times the FP32 scatter with each and keeps the
  * fastest.  A plan that does not fix the lanes may sum from a sliced layout instead (eight
- * pixels of four lanes per warp), chosen by the samples per pixel and the sizes; the number
- * given here then belongs to the scatters that it does not replace.  lanes_per_pixel (host),
- * ms (host float[3]: the timed launches for 32, 16 and
- * 8 lanes, or 0 when not timed); either may be NULL.  The paper has no counterpart.
+ * pixels of four lanes per warp), chosen by the samples per pixel and the sizes, or in FP32
+ * timed against the lanes when autotuning; mm_scatter_form tells which, and the number given
+ * here belongs to the scatters that are not sliced.  lanes_per_pixel (host), ms (host
+ * float[3]: the timed launches for 32, 16 and 8 lanes, or 0 when not timed); either may be
+ * NULL.  The paper has no counterpart.
  */
 mm_status mm_scatter_config(mm_plan_t plan, int32_t* lanes_per_pixel, float* ms);
+
+/*
+ * Form of the scatter of one right-hand side in `precision`: lanes = 4 for the sliced layout,
+ * with warps = warps that share a slice of eight pixels (1 to 32), else the lanes of
+ * mm_scatter_config and warps = 0.  Host pointers, either may be NULL.  The paper has no
+ * counterpart.
+ */
+mm_status mm_scatter_form(mm_plan_t plan, int precision, int32_t* lanes, int32_t* warps);
 
 /*
  * Form of the batched operator (mm_apply_A_batch, mm_solve_batch), fixed once per plan by

@@ -604,11 +604,13 @@ static void free_sliced(Plan& P) {
     P.sl_ang = nullptr;
 }
 
-// Frees the sorted weights that the 32-lane scatters no longer read.
+// Frees the sorted weights that no 32-lane scatter reads.
 static void free_sorted_weights(Plan& P) {
     if (P.sl_off == nullptr) return;
-    dfree(P.wsort64);
-    P.wsort64 = nullptr;
+    if (P.sl_f64) {
+        dfree(P.wsort64);
+        P.wsort64 = nullptr;
+    }
     if (!P.sl_f32) return;
     dfree(P.wsort32);
     dfree(P.asort32);
@@ -618,13 +620,10 @@ static void free_sorted_weights(Plan& P) {
 
 // The sliced layout of the scatter, unless its padding (a slice is as long as its longest
 // pixel, in fours) costs more than half as many entries again: its time is its bytes, the
-// 32-lane form's is about twice that (scatter.cu), so up to there it is ahead.  The FP32
-// scatter of one right-hand side keeps the 32-lane form while its pixels have 128 to 4095
-// samples (four or more loads a lane in flight, not many in a row) and the time-domain array
-// fits the L2 cache (I/Q/U: 47.6 us against 52.8 on 65536 pixels of 256 samples; T: 26.2
-// against 28.2 on 49000 of 256), and in small I/Q/U plans, where a slice's longer walk shows
-// (5.6 against 7.5 us on 1024 pixels of 256).
-static void build_sliced(Plan& P) {
+// 32-lane form's is about twice that for short pixels, so up to there it is ahead; or unless it
+// takes more than a quarter of the memory that is free.  tune: for the FP32 scatter of one
+// right-hand side whatever scatter_sliced says.
+static void build_sliced(Plan& P, bool tune) {
     constexpr int PIX = 8;
     if (P.npix_obs == 0) return;
     const int32_t ns = (P.npix_obs + PIX - 1) / PIX;
@@ -641,9 +640,13 @@ static void build_sliced(Plan& P) {
     }
     P.sl_count = ns;
     P.sl_steps = steps;
-    const int64_t hits = P.nkept / P.npix_obs;
-    P.sl_f32 = hits >= 4096 || P.nt > (1 << 25) || (hits < 128 && P.nkept >= (1 << 20)) || (P.ncomp == 1 && P.nkept < (1 << 20));
+    const double padded = (double)used / (double)P.npix_obs;
+    P.sl_f64 = scatter_sliced(P.ncomp, 8, P.nt, P.nkept, P.npix_obs, padded);
+    P.sl_f32 = tune || scatter_sliced(P.ncomp, 4, P.nt, P.nkept, P.npix_obs, padded);
     const size_t e = (size_t)steps * 32 + SL_PAD;
+    size_t room = 0, total = 0;
+    check_cuda(cudaMemGetInfo(&room, &total), "cudaMemGetInfo");
+    if (e * (P.ncomp == 3 ? 32 : 4) > room / 4) return;
     try {
         P.sl_off = dalloc<int32_t>(off.size());
         h2d(P.sl_off, off.data(), off.size() * 4, P.stream);
@@ -903,7 +906,7 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
         P.scatter_lpp = o->scatter_lanes;
     }
     // the sliced scatter, unless a lane count was asked for
-    if (o->scatter_lanes == 0 && !P.autotune) build_sliced(P);
+    if (o->scatter_lanes == 0 && !P.autotune) build_sliced(P, false);
     if (P.autotune) {
         // zero maps for the timed launches (x64 / the first half of r64 as FP32)
         check_cuda(cudaMemsetAsync(P.x64, 0, (size_t)P.n * 8, s), "memset");
@@ -923,11 +926,14 @@ static void build_plan(PlanHolder& P, const int32_t* pix, int64_t nt, int32_t np
                 if (P.tuned_scatter_ms[i] < P.tuned_scatter_ms[best]) best = i;
             }
             P.scatter_lpp = lpp[best];
-            build_sliced(P);
-            if (P.sl_off != nullptr && P.sl_f32)
-                P.sl_f32 = time_launches(
-                               P, [&] { launch_scatter<float>(P, P.tod32, reinterpret_cast<float*>(P.r64), nullptr, s); },
-                               5) <= P.tuned_scatter_ms[best];
+            build_sliced(P, true);
+            if (P.sl_off != nullptr &&
+                time_launches(P, [&] { launch_scatter<float>(P, P.tod32, reinterpret_cast<float*>(P.r64), nullptr, s); }, 5) >
+                    P.tuned_scatter_ms[best]) {
+                P.sl_f32 = false;
+                dfree(P.sl_ang);
+                P.sl_ang = nullptr;
+            }
         }
     }
     free_sorted_weights(P);
@@ -2768,6 +2774,15 @@ mm_status mm_scatter_config(mm_plan_t plan, int32_t* lanes_per_pixel, float* ms)
         PlanHolder* P = get(plan);
         if (lanes_per_pixel) *lanes_per_pixel = P->scatter_lpp;
         if (ms) std::memcpy(ms, P->tuned_scatter_ms, sizeof(P->tuned_scatter_ms));
+    });
+}
+
+mm_status mm_scatter_form(mm_plan_t plan, int precision, int32_t* lanes, int32_t* warps) {
+    return guarded(plan, [&] {
+        PlanHolder* P = get(plan);
+        const bool sliced = prec_ok(precision) == MM_FP64 ? use_sliced<double>(*P) : use_sliced<float>(*P);
+        if (lanes) *lanes = sliced ? 4 : P->scatter_lpp;
+        if (warps) *warps = sliced ? sliced_parts(*P) : 0;
     });
 }
 

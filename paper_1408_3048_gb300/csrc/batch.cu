@@ -297,7 +297,12 @@ __global__ void batch_scatter_kernel(const int32_t* __restrict__ off, const int3
 
 void launch_batch_scatter(const Plan& P, const float* Z, float* W, int R, const int* done, cudaStream_t s) {
     if (P.npix_obs == 0) return;
-    if (P.sl_off != nullptr) return launch_batch_scatter_sliced<float>(P, Z, W, R, done, s);
+    // up to three columns as one (scatter_sliced; I/Q/U, 4096 pixels of 1024 samples, A x in us, this
+    // form against the sliced one: R = 1 72 : 90, 2 107 : 123, 3 135 : 156, 4 164 : 175, 8 278 : 254;
+    // of 256 samples R = 3 131 : 132, 4 158 : 156); few pixels leave this form's warps idle (1024 of
+    // 2048 samples, two columns 76 : 68, 64 of 8192 119 : 74)
+    if (P.sl_off != nullptr && (R > 3 || P.sl_f32 || P.npix_obs <= 1024))
+        return launch_batch_scatter_sliced<float>(P, Z, W, R, done, s);
     const int th = 256;
     int g = (P.npix_obs + 7) / 8;
     if (g > P.num_sms * 32) g = P.num_sms * 32;

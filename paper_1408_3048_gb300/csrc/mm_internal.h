@@ -154,8 +154,9 @@ struct Plan {
                                    // pair has unit norm (the FP32 scatter reads 4 bytes, not 8)
     // sliced layout of the sorted samples (scatter.cu), or null: slices of eight pixels, step j
     // of a slice = 32 entries (four samples of each of its pixels); the sorted weight arrays
-    // above that no scatter reads any more are then freed once the plan is built
-    bool sl_f32 = false;           // the FP32 scatter of one right-hand side uses it too
+    // above that no scatter reads any more are then freed once the plan is built.  Batches of
+    // four or more use it, smaller ones as the FP32 scatter of one right-hand side.
+    bool sl_f64 = false, sl_f32 = false;   // the scatters of one right-hand side use it
     int32_t sl_count = 0;          // slices
     int64_t sl_steps = 0;          // steps in all
     int32_t* sl_off = nullptr;     // [sl_count + 1] first step
@@ -268,6 +269,7 @@ void fold_split_spectrum(const std::vector<double>& h, int64_t N, const std::vec
 // per-pass Stockham twiddles of an N = 2^logn point FFT as interleaved (cos, sin)
 std::vector<double> pass_twiddle_table(int logn);
 double rcond_sym3(const double B[6]);
+bool scatter_sliced(int ncomp, int bytes, int64_t nt, int64_t nkept, int64_t npix, double padded);
 
 // kernels (launchers) --------------------------------------------------------------------
 // Toeplitz overlap-save (toeplitz_f64.cu / toeplitz_f32.cu)
@@ -315,6 +317,9 @@ template <typename T>
 void launch_scatter_dot(const Plan& P, const T* z, T* w, const T* p, double* part, unsigned* count, double* pq,
                         const int* done, cudaStream_t s);
 int scatter_blocks(const Plan& P);
+// whether launch_scatter<T> sums from the sliced layout
+template <typename T>
+bool use_sliced(const Plan& P) { return P.sl_off != nullptr && (sizeof(T) == 8 ? P.sl_f64 : P.sl_f32); }
 // the same from the sliced layout (P.sl_off != nullptr); p null: no dot product
 void launch_slice_fill(const Plan& P, int32_t* st, double2* sw64, float2* sw32, float* sang, cudaStream_t s);
 template <typename T>
@@ -322,6 +327,7 @@ void launch_scatter_sliced(const Plan& P, const T* z, T* w, const T* p, double* 
                            const int* done, cudaStream_t s);
 template <typename T>
 void launch_batch_scatter_sliced(const Plan& P, const T* Z, T* W, int R, const int* done, cudaStream_t s);
+int sliced_parts(const Plan& P, int groups = 0);   // warps per slice; groups of a batch, 0: one column
 void launch_bd_build(const Plan& P, double* bd64, float* bd32, cudaStream_t s);
 // merged a priori coarse space Z_S (Sec. 3.3.1), r groups of consecutive intervals, into
 // Z [r][n] FP64 (zeroed here)

@@ -289,9 +289,6 @@ static void scatter_launch(const Plan& P, const T* z, T* w, const int* done, Sca
 }
 
 template <typename T>
-static bool use_sliced(const Plan& P) { return P.sl_off != nullptr && (sizeof(T) == 8 || P.sl_f32); }
-
-template <typename T>
 void launch_scatter(const Plan& P, const T* z, T* w, const int* done, cudaStream_t s) {
     if (P.npix_obs == 0) return;
     if (use_sliced<T>(P)) return launch_scatter_sliced<T>(P, z, w, nullptr, nullptr, nullptr, nullptr, done, s);

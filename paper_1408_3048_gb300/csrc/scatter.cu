@@ -13,7 +13,7 @@
 // 264 -> 98 us (537 MB, 0.81 of the copy bandwidth); I/Q/U circles, 1.6e7 samples on 303079
 // pixels 99 -> 63 us; I/Q/U in FP64, 2^22 samples 106 -> 39 us; 64 right-hand sides on 2^22
 // samples 481 -> 318 us.  I/Q/U in FP32 on 65536 pixels of 256 samples: 47.6 -> 52.8 us, so
-// there the 32-lane form stays (build_sliced).
+// there the 32-lane form stays (scatter_sliced in plan_host.cpp has the rule and its figures).
 //
 // Few pixels with many samples: the S warps of a slice take consecutive parts of its steps and
 // add them in order through shared memory.  Every sum has a fixed order: bit-reproducible.
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(WPB * 32, (sl_min_blocks<T, NC, WPB>())) slice
 // sides, each a walk over every slice; a batch's warps have several loads in flight for a step
 // and fill the chip four times as early (512 slices of 64 steps, four groups of four columns:
 // one warp per slice, with two a batched solve took 2 % longer).
-static int sliced_parts(const Plan& P, int groups = 0) {
+int sliced_parts(const Plan& P, int groups) {
     const int64_t steps = P.sl_count > 0 ? P.sl_steps / P.sl_count : 0;
     const int64_t enough = (int64_t)P.num_sms * (groups > 0 ? 8 : 32), walks = (int64_t)P.sl_count * std::max(groups, 1);
     int S = 1;

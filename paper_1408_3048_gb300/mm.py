@@ -34,7 +34,7 @@ EXPORTS = ["mm_plan", "mm_plan_info", "mm_plan_pixels", "mm_plan_row", "mm_gathe
            "mm_version", "mm_launch_count", "mm_apply_A_static", "mm_solve_ex", "mm_grad", "mm_apply_A_batch",
            "mm_solve_batch", "mm_autotune_read", "mm_batch_config", "mm_build_coarse_apriori",
            "mm_build_coarse_eps", "mm_coarse_import", "mm_build_coarse_arnoldi", "mm_solve_history",
-           "mm_pcg_barrier_check", "mm_residual", "mm_scatter_config"]
+           "mm_pcg_barrier_check", "mm_residual", "mm_scatter_config", "mm_scatter_form"]
 
 
 class mm_psd(ctypes.Structure):
@@ -108,6 +108,7 @@ _SIGS = {
     "mm_pcg_barrier_check": (I32, [P, I32, ctypes.c_double]),
     "mm_residual": (I32, [P, ctypes.c_int, P, P, P]),
     "mm_scatter_config": (I32, [P, P, P]),
+    "mm_scatter_form": (I32, [P, ctypes.c_int, P, P]),
     "mm_last_error": (ctypes.c_char_p, [P]),
     "mm_destroy": (None, [P]),
     "mm_version": (ctypes.c_char_p, []),
@@ -326,6 +327,13 @@ def mm_scatter_config(plan):
     ms = (ctypes.c_float * 3)()
     _check(lib().mm_scatter_config(plan, ctypes.byref(lpp), ms), plan)
     return lpp.value, list(ms)
+
+
+def mm_scatter_form(plan, precision):
+    """(lanes per pixel, warps per slice) of the scatter: 4 lanes = the sliced layout, else 0 warps."""
+    lanes, warps = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().mm_scatter_form(plan, int(precision), ctypes.byref(lanes), ctypes.byref(warps)), plan)
+    return lanes.value, warps.value
 
 
 def mm_residual(plan, arith, d, x, r):
@@ -603,6 +611,10 @@ class Plan:
     def scatter_config(self):
         """(lanes per pixel of the scatter, timings at 32 / 16 / 8 lanes when autotuned)."""
         return mm_scatter_config(self.handle)
+
+    def scatter_form(self, precision=MM_FP64):
+        """(lanes per pixel, warps per slice) of the scatter in `precision`; 4 lanes: the sliced layout."""
+        return mm_scatter_form(self.handle, precision)
 
     def barrier_check(self, absent_blocks, wait_s):
         """Status (int) of the bounded-wait diagnostic mm_pcg_barrier_check."""

@@ -14,7 +14,7 @@
 namespace {
 std::map<char*, size_t> blocks;
 long long left = -1;            // allocations until one fails (-1: none does)
-size_t live_bytes = 0, peak_bytes = 0;
+size_t live_bytes = 0, peak_bytes = 0, room_bytes = size_t(270) << 30;
 std::map<const void*, std::string> names;
 cudaError_t last = cudaSuccess;
 struct Launch {
@@ -68,6 +68,7 @@ long long fake_peak_bytes(int reset) {
     if (reset) peak_bytes = live_bytes;
     return (long long)peak_bytes;
 }
+void fake_room(long long bytes) { room_bytes = (size_t)bytes; }   // free memory that is reported
 void fake_clear_launches() { launches.clear(); }
 int fake_launches() { return (int)launches.size(); }
 const char* fake_launch_name(int i) { return launches[(size_t)i].name.c_str(); }
@@ -120,6 +121,11 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, 
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
     if (d == nullptr) return set(cudaErrorInvalidValue);
     std::memset(d, v, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemGetInfo(size_t* room, size_t* total) {
+    *total = size_t(280) << 30;
+    *room = room_bytes;
     return cudaSuccess;
 }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {

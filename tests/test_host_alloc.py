@@ -36,7 +36,7 @@ def load(so):
         fn.restype, fn.argtypes = res, args
     for name in ("fake_live_bytes", "fake_peak_bytes"):
         getattr(L, name).restype = ctypes.c_longlong
-    L.fake_fail_after.argtypes = [ctypes.c_longlong]
+    L.fake_fail_after.argtypes = L.fake_room.argtypes = [ctypes.c_longlong]
     L.fake_launch_name.restype = ctypes.c_char_p
     return L
 
@@ -214,3 +214,37 @@ def test_batched_scatter_of_few_pixels_fills_the_chip(lib):
     name, blocks, _ = p.batch(4)[1][-1]
     assert "sliced_batch_parts_kernelIfLi3ELi4ELi8E" in name and blocks == 512 // 4
     p.close()
+
+
+def scatters(L, p):
+    """(FP64, FP32) forms of the plan, and the kernels that its scatters launch."""
+    forms, names, v = [], [], np.zeros(max(p.nt, p.n))
+    for prec in (mm.MM_FP64, mm.MM_FP32):
+        lanes, warps = ctypes.c_int32(), ctypes.c_int32()
+        assert L.mm_scatter_form(p.h, prec, ctypes.byref(lanes), ctypes.byref(warps)) == mm.MM_OK
+        forms.append((lanes.value, warps.value))
+        L.fake_clear_launches()
+        assert L.mm_scatter(p.h, prec, v.ctypes.data, v.ctypes.data) == mm.MM_OK
+        (name, _, _), = launches(L)
+        names.append("sliced" if "sliced_scatter" in name else "lanes")
+    return forms, names
+
+
+def test_scatter_form_by_samples_and_memory(lib):
+    for side, ncomp, want in ((32, 3, ["lanes", "lanes"]), (64, 3, ["sliced", "lanes"]), (128, 3, ["sliced", "sliced"]),
+                              (32, 1, ["lanes", "lanes"]), (14, 1, ["lanes", "sliced"]), (8, 1, ["sliced", "sliced"])):
+        p = Plan(lib, [1 << 19], 100, ncomp, side=side)   # 1024, 256, 64, 1024, 5349 and 16384 samples per pixel
+        forms, names = scatters(lib, p)
+        assert names == want and [f[0] for f in forms] == [4 if n == "sliced" else 32 for n in names], side
+        for R in (2, 4):   # a small batch goes as one column does
+            name = p.batch(R)[1][-1][0]
+            assert ("sliced_batch" in name) == (R > 3 or names[1] == "sliced" or side <= 32), (side, R, name)
+        p.close()
+    # the layout takes a quarter of the free memory at most: 32 bytes for each of 2^20 samples
+    for room, want in ((120 << 20, "lanes"), (140 << 20, "sliced")):
+        lib.fake_room(room)
+        p = Plan(lib, [1 << 19], 100, 3, side=128)
+        assert scatters(lib, p)[1] == [want] * 2
+        assert p.batch(4)[0] == mm.MM_OK
+        p.close()
+    lib.fake_room(270 << 30)
