@@ -2309,7 +2309,7 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
         launch_toeplitz_any<float>(P, batch_tz(P, Rc), nullptr, Dg, nullptr, Rc, (int64_t)nt, bt.tod, (int64_t)nt, nullptr, s);
         launch_batch_scatter(P, bt.tod, bt.z, Rc, nullptr, s);
         launch_convert_f32_to_f64(bt.z, bt.b64, (int64_t)Rc * n, s);
-        launch_dot_batch(bt.b64, (int64_t)n, Rc, bt.scal, s);
+        launch_dot_batch(bt.b64, (int64_t)n, Rc, P.d_dot, bt.scal, s);
         d2h(bb.data(), bt.scal, (size_t)Rc * 8, s);
         sync(P);
         rr = bb;
@@ -2355,7 +2355,7 @@ static void solve_batch(PlanHolder& P, const double* D, int R, const mm_solve_op
             launch_axpy_f32_batch(bt.x64, bt.x, bt.scal, (int64_t)n, Rc, s);
             residual64_batch(P, Dg, nrm, active, Rc, so.residual != MM_RESID_FP64);
             std::vector<double> now((size_t)Rc);
-            launch_dot_batch(bt.r64, (int64_t)n, Rc, bt.scal, s);
+            launch_dot_batch(bt.r64, (int64_t)n, Rc, P.d_dot, bt.scal, s);
             d2h(now.data(), bt.scal, (size_t)Rc * 8, s);
             sync(P);
             for (int r = 0; r < Rc; ++r)

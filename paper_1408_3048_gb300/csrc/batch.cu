@@ -569,22 +569,37 @@ __global__ void axpy_f32_batch_kernel(double* __restrict__ x, const float* __res
         x[o + i] += s * (double)d[o + i];
 }
 
-// out[r] = a_r . a_r: one block per column, a fixed order of sums
-__global__ void __launch_bounds__(1024) dot_batch_kernel(const double* __restrict__ a, int64_t n, double* __restrict__ out) {
+// Sum over the block in a fixed order, valid in thread 0.
+__device__ __forceinline__ double dot_block_sum(double s) {
     __shared__ double sh[32];
-    const double* v = a + (int64_t)blockIdx.x * n;
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += v[i] * v[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x < 32) {
-        s = sh[threadIdx.x];
+        s = threadIdx.x < blockDim.x >> 5 ? sh[threadIdx.x] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) out[blockIdx.x] = s;
     }
+    return s;
+}
+
+// part[r][b] = block b's share of a_r . a_r (grid: blocks, columns); with one block a column the
+// sum itself
+__global__ void __launch_bounds__(1024) dot_batch_kernel(const double* __restrict__ a, int64_t n, double* __restrict__ part) {
+    const double* v = a + (int64_t)blockIdx.y * n;
+    double s = 0.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        s += v[i] * v[i];
+    s = dot_block_sum(s);
+    if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
+}
+
+__global__ void dot_batch_sum_kernel(const double* __restrict__ part, int blocks, double* __restrict__ out) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < blocks; i += blockDim.x) s += part[(int64_t)blockIdx.x * blocks + i];
+    s = dot_block_sum(s);
+    if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 static dim3 batch_grid(int64_t n, int R) {
@@ -605,10 +620,15 @@ void launch_axpy_f32_batch(double* x, const float* d, const double* sc, int64_t 
     note_launch();
 }
 
-void launch_dot_batch(const double* a, int64_t n, int R, double* out, cudaStream_t st) {
-    dot_batch_kernel<<<R, 1024, 0, st>>>(a, n, out);
+// Two blocks per SM over all columns, each with 16 values a thread or more: one block a column
+// took 517 us for two columns of 2.1e6 values, this 18; columns of less than 32768 values take
+// one (the second launch costs 3).
+void launch_dot_batch(const double* a, int64_t n, int R, double* part, double* out, cudaStream_t st) {
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(DOT_BLOCKS / R, n / 16384));
+    dot_batch_kernel<<<dim3((unsigned)blocks, (unsigned)R), 1024, 0, st>>>(a, n, blocks > 1 ? part : out);
+    if (blocks > 1) dot_batch_sum_kernel<<<R, 128, 0, st>>>(part, blocks, out);
     check_cuda(cudaGetLastError(), "dot launch");
-    note_launch();
+    note_launch(blocks > 1 ? 2 : 1);
 }
 
 }  // namespace mm

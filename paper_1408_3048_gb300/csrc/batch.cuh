@@ -86,8 +86,8 @@ int batch_pcg_max_blocks(int num_sms);
 }  // namespace mm
 
 namespace mm {
-// R columns of n values; sc, out: device double[R]
+// R columns of n values; sc, out: device double[R], part: device double[DOT_BLOCKS] (pcg.cuh)
 void launch_scale_f32_batch(const double* a, const double* sc, float* out, int64_t n, int R, cudaStream_t st);
 void launch_axpy_f32_batch(double* x, const float* d, const double* sc, int64_t n, int R, cudaStream_t st);
-void launch_dot_batch(const double* a, int64_t n, int R, double* out, cudaStream_t st);
+void launch_dot_batch(const double* a, int64_t n, int R, double* part, double* out, cudaStream_t st);
 }  // namespace mm

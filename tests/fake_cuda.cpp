@@ -43,7 +43,7 @@ void record(const void* f, dim3 grid, void** args) {
     auto word = [&](int arg, int at) { return *reinterpret_cast<void**>(static_cast<char*>(args[arg]) + 8 * at); };
     if (l.name.find("toeplitz_ws") != std::string::npos) l.ptrs = {word(0, 0), word(4, 0), word(5, 0), word(6, 0)};
     else if (l.name.find("toeplitz_os") != std::string::npos) l.ptrs = {word(0, 0), word(0, 3)};
-    else if (l.name.find("dot_batch") != std::string::npos) l.ptrs = {word(0, 0), word(2, 0)};
+    else if (l.name.find("dot_batch_kernel") != std::string::npos) l.ptrs = {word(0, 0), word(2, 0)};
     launches.push_back(l);
 }
 

@@ -248,3 +248,12 @@ def test_scatter_form_by_samples_and_memory(lib):
         assert p.batch(4)[0] == mm.MM_OK
         p.close()
     lib.fake_room(270 << 30)
+
+
+def test_batched_dot_products_use_the_chip(lib):
+    """Two columns of 10^5 values: several blocks for each; many small columns: one each."""
+    for side, R, want in ((180, 2, 2 * (3 * 180 * 180 // 16384)), (400, 2, 2 * (3 * 400 * 400 // 16384)), (16, 5, 5)):
+        p = Plan(lib, [4 * side * side], 50, 3, side=side)
+        dots = [grid for name, grid, _ in p.solve_batch(R)[1] if "dot_batch_kernel" in name]
+        assert dots == [want], side
+        p.close()
