@@ -156,32 +156,51 @@ def peaks():
 ALU_PEAK = {"f64": 1.25e12, "f32": 152 * 128 * 2 * 2.07e9}
 
 
-def fft_tiles(scan, B, max_segments=3):
+def fft_tiles(scan, B, max_segments=3, fours=False):
     """Overlap-save tiles of B-sample blocks as the plan lays them out: consecutive
     intervals with the same PSD are packed into one sequence with lambda zeros between
     them when that needs fewer tiles (and no tile holds more than `max_segments`
-    intervals), else every interval is tiled on its own."""
+    intervals), else every interval is tiled on its own.  fours: blocks of the persistent
+    FP32 kernel, whose tiles have a multiple of four outputs and whose intervals start at
+    times that differ from their positions by one, unless that takes over a fifth more."""
     lam = int(scan.lam)
-    Lv = B - 2 * lam
-    lens = np.diff(np.asarray(scan.offsets, dtype=np.int64))
-    psd = np.asarray(getattr(scan, "interval_psd", np.arange(lens.size)))
+    off = np.asarray(scan.offsets, dtype=np.int64)
+    psd = np.asarray(getattr(scan, "interval_psd", np.arange(off.size - 1)))
+
+    def run(i0, i1, fours):
+        Lv = B - 2 * lam
+        if fours and Lv >= 4:
+            Lv -= Lv % 4
+
+        def lay_out(j0, j1):   # virtual start of each interval, length of the sequence
+            starts, vlen = [], 0
+            for i in range(j0, j1):
+                vlen += lam if i > j0 else 0
+                vlen += int(off[i] - lam - vlen) % 4 if fours else 0
+                starts.append(vlen)
+                vlen += int(off[i + 1] - off[i])
+            return np.array(starts), vlen
+        single = sum(-(-lay_out(i, i + 1)[1] // Lv) for i in range(i0, i1))
+        starts, vlen = lay_out(i0, i1)
+        packed = -(-vlen // Lv)
+        if i1 - i0 == 1 or packed >= single:
+            return single
+        ends = starts + off[i0 + 1:i1 + 1] - off[i0:i1]
+        for w0 in range(-lam, packed * Lv - lam, Lv):
+            if np.sum((starts < w0 + B) & (ends > w0)) > max_segments:
+                return single
+        return packed
+
     total, i0 = 0, 0
-    while i0 < lens.size:
+    while i0 < off.size - 1:
         i1 = i0 + 1
-        while i1 < lens.size and psd[i1] == psd[i0]:
+        while i1 < off.size - 1 and psd[i1] == psd[i0]:
             i1 += 1
-        single = int(np.sum((lens[i0:i1] + Lv - 1) // Lv))
-        starts = np.concatenate([[0], np.cumsum(lens[i0:i1] + lam)[:-1]])
-        vlen = int(lens[i0:i1].sum() + (i1 - i0 - 1) * lam)
-        packed = (vlen + Lv - 1) // Lv
-        ok = True
-        for k in range(packed):
-            w0 = k * Lv - lam
-            seg = np.sum((starts < w0 + B) & (starts + lens[i0:i1] > w0))
-            if seg > max_segments:
-                ok = False
-                break
-        total += packed if (i1 - i0 > 1 and ok and packed < single) else single
+        n = run(i0, i1, False)
+        if fours:
+            n4 = run(i0, i1, True)
+            n = n4 if 5 * n4 <= 6 * n else n
+        total += n
         i0 = i1
     return total
 
@@ -244,7 +263,7 @@ def roofline(kernel, ms, plan, scan, hbm, peak_src):
         byts = ax_bytes(plan, s)
         B = plan.fft_block_f32 if key == "f32" else plan.fft_block_f64
         N = B // 2
-        tiles = fft_tiles(scan, B)
+        tiles = fft_tiles(scan, B, fours=key == "f32" and B in (1 << 14, 1 << 15))
         # two N-point complex FFTs (5 N log2 N each), real-FFT split/merge and spectrum
         # product (20 N), I/Q/U de-pointing (2 FMA per sample)
         flops = tiles * (2 * 5 * N * np.log2(N) + 20 * N) + (4 * nt if plan.ncomp == 3 else 0)

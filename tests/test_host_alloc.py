@@ -7,6 +7,7 @@ import os
 import shutil
 import subprocess
 import sys
+from types import SimpleNamespace
 
 import numpy as np
 import pytest
@@ -257,3 +258,24 @@ def test_batched_dot_products_use_the_chip(lib):
         dots = [grid for name, grid, _ in p.solve_batch(R)[1] if "dot_batch_kernel" in name]
         assert dots == [want], side
         p.close()
+
+
+@pytest.mark.parametrize("lengths,lam,log2B", [([9001, 20003, 4999], 511, 14), ([14382, 14382], 1001, 14), ([3000, 2999, 5001], 101, 15),
+                                              ([40001], 4095, 15), ([700] * 9, 64, 14), ([2094] * 5, 1001, 12),
+                                              ([30000, 30001, 9999], 2047, 14)])
+def test_bench_counts_the_plans_tiles(lib, lengths, lam, log2B):
+    """bench.fft_tiles (its roofline's operations) against the launches' grids, in both layouts."""
+    import bench
+    p = Plan(lib, lengths, lam, 1, fft_log2_f64=log2B, fft_log2_f32=log2B)
+    v = np.zeros(p.nt)
+    scan = SimpleNamespace(lam=lam, offsets=np.concatenate([[0], np.cumsum(list(lengths) * 2)]),
+                           interval_psd=np.repeat([0, 1], len(lengths)))
+    for prec in (mm.MM_FP64, mm.MM_FP32):
+        lib.fake_clear_launches()
+        assert lib.mm_apply_ninv(p.h, prec, v.ctypes.data, v.ctypes.data) == mm.MM_OK
+        (name, grid, _), = launches(lib)
+        fours = "toeplitz_ws" in name
+        assert fours == (prec == mm.MM_FP32 and log2B >= 14)
+        ctas = 2 if "oscl" in name else 1   # per tile: two-CTA clusters; the persistent kernel: one tile each here
+        assert grid == ctas * bench.fft_tiles(scan, 1 << log2B, fours=fours)
+    p.close()
