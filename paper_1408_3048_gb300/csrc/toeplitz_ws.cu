@@ -6,10 +6,11 @@
 // threads (one 136 KB block per SM) neither uses what the other leaves idle: the gather took
 // 40 % of a block's time, transforms and product 49 %, stores 11 %.  Here a CTA walks over its
 // blocks with two kinds of warps: the gather warps form P x of the next block into a scratch
-// buffer of the CTA (two of B floats in global memory, which stay in L2) while the transform
-// warps work on the current one; one CTA-wide barrier per block swaps them.  A CTA's blocks
-// are consecutive windows, so the 2 lambda positions that two windows share are copied from
-// buffer to buffer instead of gathered twice.
+// buffer of the CTA (two of B floats in global memory, read back through L2, which writes most
+// of them to memory all the same: 127 MB of DRAM writes a launch, 67 of them output) while the
+// transform warps work on the current one; one CTA-wide barrier per block swaps them.  A CTA's
+// blocks are consecutive windows: where their distance is a multiple of four, the 2 lambda
+// positions that two windows share are copied from buffer to buffer instead of gathered twice.
 //
 // Measured (I/Q/U, 2^24 samples, lambda = 4096, 736 blocks): 153 -> 118 us, of which 11 us are
 // the first block's gather (nothing to overlap it with); per block 38k cycles of transform,
