@@ -737,8 +737,8 @@ __device__ __forceinline__ void split_chain(typename Cx<T>::type u1, typename Cx
 // f_knee = 1 to 2 Hz the FP64 product left 3e-15 to 1e-12 of the lowest modes as rounding, the
 // chain less than 2e-15.  So FP32 takes the chain throughout, FP64 and double-float for the
 // bins where H_k and H_{N-k} differ by more than a factor 1 / SPLIT_RATIO (f_knee = 2 Hz at 100
-// Hz: 1 bin in 20; A x of 2^22 I/Q/U samples 808 -> 813 us, the double-float residual
-// unchanged at 481).
+// Hz: 1 bin in 20; A x of 2^22 I/Q/U samples 808 -> 809 us, the double-float residual
+// 476 -> 473).
 template <typename T>
 __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename Cx<T>::type u2, T a1, T a2, T b,
                                               typename Cx<T>::type& V1, typename Cx<T>::type& V2) {
@@ -755,19 +755,23 @@ template <typename T, int N>
 struct SplitRow {
     const T *al, *be, *quarter;
     int kc;
-    __device__ __forceinline__ SplitRow(const T* row, const T* q) : al(row), be(row + N), quarter(q) {
-        const T v = be[N / 2 + 1];
-        if constexpr (std::is_same<T, double>::value) kc = (int)v;
-        else kc = (int)v.hi;
+    __device__ __forceinline__ SplitRow(const T* row, const T* q, int chained)
+        : al(row), be(row + N), quarter(q), kc(chained) {}
+    // bins that go through the chain: read ahead of the transform, as the branch waits for it
+    static __device__ __forceinline__ int chained(const T* row) {
+        const T v = row[N + N / 2 + 1];
+        if constexpr (std::is_same<T, double>::value) return (int)v;
+        else return (int)v.hi;
     }
     __device__ __forceinline__ void product(typename Cx<T>::type u1, typename Cx<T>::type u2, int k, T a1, T a2,
                                             typename Cx<T>::type& V1, typename Cx<T>::type& V2) const {
         const int m = k <= N / 2 ? k : N - k;
+        const T b = be[m];   // requested with the others, ahead of the branch
         if (m < kc) {
             const T c = quarter[m];
-            split_chain<T>(u1, u2, k <= N / 2 ? c : -c, quarter[N / 2 - m], a1, k == 0 ? be[0] : a2, V1, V2);
+            split_chain<T>(u1, u2, k <= N / 2 ? c : -c, quarter[N / 2 - m], a1, k == 0 ? b : a2, V1, V2);
         } else {
-            split_product<T>(u1, u2, a1, a2, be[m], V1, V2);
+            split_product<T>(u1, u2, a1, a2, b, V1, V2);
         }
     }
 };
@@ -788,6 +792,8 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
     PfSeg next{0, 0, 0};
     if (A.pf_ahead > 0 && (int64_t)blockIdx.x + A.pf_ahead < (int64_t)gridDim.x)
         next = prefetch_seg(A, blockIdx.x + A.pf_ahead, threadIdx.x);
+    int kc = 0;
+    if constexpr (sizeof(T) != 4) kc = SplitRow<T, N>::chained(A.H + tile.psd * split_size(N));
     load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), 0, 2 * N, tr.rhs);
     __syncthreads();
     prefetch_issue<T, MODE>(A, next);
@@ -819,7 +825,7 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
         }
         if (tid == 0) product(N / 2, __ldg(H + N / 2), __ldg(H + N / 2));
     } else {
-        const SplitRow<T, N> row(A.H + tile.psd * split_size(N), A.twiddle);
+        const SplitRow<T, N> row(A.H + tile.psd * split_size(N), A.twiddle, kc);
         for (int k = tid; k <= N / 2; k += NT) {
             const int k2 = (N - k) & (N - 1);
             C2 V1, V2;
@@ -920,6 +926,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     const TileRhs tr = tile_rhs(blockIdx.x / CL, A.R);
     const Tile tile = A.tiles[tr.tile];
     const int tid = threadIdx.x;
+    int kc = 0;
+    if constexpr (sizeof(T) != 4) kc = SplitRow<T, N>::chained(A.H + tile.psd * split_size(N));
     load_block<T, NT, MODE>(A, tile, reinterpret_cast<T*>(a), rank * 2 * M, 2 * M, tr.rhs);
     cl.sync();
     C2 y[PER];
@@ -950,9 +958,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT) toeplitz_oscl_k
     const T* al = A.H + tile.psd * HS;
     // bins k and N - k (FP32: the chain, al = the spectrum itself, h1 and h2 its values)
     struct NoRow {
-        __device__ NoRow(const T*, const T*) {}
+        __device__ NoRow(const T*, const T*, int) {}
     };
-    const typename std::conditional<F32, NoRow, SplitRow<T, N>>::type row(al, A.twiddle);
+    const typename std::conditional<F32, NoRow, SplitRow<T, N>>::type row(al, A.twiddle, kc);
     auto product = [&](C2 u1, C2 u2, int k, T h1, T h2, C2& V1, C2& V2) {
         if constexpr (F32) {
             float sw, cw;
