@@ -265,19 +265,26 @@ __global__ void batch_scatter_kernel(const int32_t* __restrict__ off, const int3
         const int e = off[q + 1];
         for (int r = 0; r < R; ++r) {
             const float* z = Z + (size_t)r * nt;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-            for (int j = b + lane; j < e; j += 32) {
-                const float v = z[tsort[j]];
-                a0 += v;
+            // FP32 pairs, to which sums of eight are added, and exact pair trees over the warp (FP64
+            // sums per pixel and RHS would make this kernel FP64-bound on GB300)
+            float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
+            for (int j = b + lane; j < e;) {
+                float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+                for (const int j1 = min(e, j + 256); j < j1; j += 32) {
+                    const float v = z[tsort[j]];
+                    a0 += v;
+                    if constexpr (NC == 3) {
+                        const float2 ww = ws[j];
+                        a1 += ww.x * v;
+                        a2 += ww.y * v;
+                    }
+                }
+                pair_add(h0, l0, a0, 0.f);
                 if constexpr (NC == 3) {
-                    const float2 ww = ws[j];
-                    a1 += ww.x * v;
-                    a2 += ww.y * v;
+                    pair_add(h1, l1, a1, 0.f);
+                    pair_add(h2, l2, a2, 0.f);
                 }
             }
-            // exact FP32-pair warp trees (FP64 shuffles per pixel and RHS would make
-            // this kernel FP64-bound on GB300)
-            float h0 = a0, l0 = 0.f, h1 = a1, l1 = 0.f, h2 = a2, l2 = 0.f;
             warp_pair_reduce(h0, l0);
             if constexpr (NC == 3) {
                 warp_pair_reduce(h1, l1);

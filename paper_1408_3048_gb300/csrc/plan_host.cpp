@@ -193,27 +193,32 @@ void fold_split_spectrum(const std::vector<double>& h, int64_t N, const std::vec
 // 2^16 .. 2^27 samples, 6 .. 16384 per pixel, rasters and circles, T and I/Q/U (times in us,
 // CSR : sliced).  The sliced walk has no tree over a pixel's lanes, which is what short pixels
 // cost; the CSR form keeps more loads in flight once a pixel has several for each lane.
-//   short     few samples per pixel, padding counted: FP32 T 2^22 samples of 64 per pixel 15.9 : 9.6,
+//   short     few samples per pixel (T: padding counted): FP32 T 2^22 samples of 64 per pixel 15.9 : 9.6,
 //             128 11.7 : 9.7, circles of 141 (155 padded) at 2^24 41 : 50; I/Q/U 2^24 96 65 : 47,
-//             128 at 2^20 7.7 : 9.7, circles of 136 (150) at 2^22 18.6 : 22.2; with fewer samples in
+//             128 at 2^20 7.7 : 9.7, circles of 136 at 2^22 18.6 : 22.2; with fewer samples in
 //             all only the shortest gain (2^18 16 8.7 : 5.6, 48 6.7 : 7.7; I/Q/U 2^18 16 9.7 : 7.7,
 //             64 7.7 : 7.9).  FP64 2^22 128 T 26 : 20, I/Q/U 63 : 43, 256 20 : 20, 49 : 40, 400
 //             18 : 21, 46 : 49, 1024 18 : 22, 39 : 49; circles of 279 20 : 22, 49 : 56.
-//   few       pixels, long ones, where the CSR form has too few warps: FP32 I/Q/U 784 pixels of 5349
-//             30 : 18, 1024 of 16384 90 : 49; T 49 of 5349 17.9 : 11.8; but I/Q/U 49 of 5349 20 : 24 on
-//             scattered pixels, 3249 of 5163 46 : 59, circles 6000 pixels 113 : 176.  FP64 I/Q/U 784 of
-//             5349 100 : 58, 196 53 : 57, 3249 116 : 182; T 1024 of 16384 100 : 57, 784 of 5349 25 : 24.
+//   few       pixels, long ones, where the CSR form has too few warps: FP32 T 49 of 5349 17.9 : 11.8,
+//             3249 of 5163 41 : 57, circles 6000 pixels 88 : 140.  FP64 I/Q/U 784 of 5349 100 : 58, 196
+//             53 : 57, 3249 116 : 182; T 1024 of 16384 100 : 57, 784 of 5349 25 : 24.
 //   long      runs whose time-domain array exceeds the L2 cache, which the CSR form reads in as
 //             many places as a pixel has visits: FP32 2^26 samples, raster of 256 T 259 : 96, I/Q/U
-//             290 : 140, circles of 141 231 : 118, 294 : 159; but of 558 123 : 166, 187 : 224, of
-//             1092 140 : 207; 2^27 circles of 558 332 : 271, 495 : 349.  FP64 2^26, raster of 256
-//             387 : 166, 622 : 428, circles of 1092 213 : 383, 446 : 671.
+//             290 : 140, circles of 141 231 : 118, 294 : 159; T of 558 123 : 166, of 1092 140 : 207; 2^27
+//             circles of 558 332 : 271, 495 : 349.  FP64 2^26, raster of 256 387 : 166, 622 : 428,
+//             circles of 1092 213 : 383, 446 : 671.
+// FP32 I/Q/U pixels of 4096 and more samples and all of 2^25 and more in all are sliced, few and
+// long or not: the CSR form forms its weights by the fast sine and cosine and adds a lane's share
+// plainly, which costs accuracy there (5000 samples 2.6e-7 of a scatter, sliced 6.9e-8); as
+// accurate it takes 63 : 59 (raster of 5163, 2^24), 187 : 158 (1024, 2^26), 163 : 176 (circles of
+// 9633, 2^25).
 bool scatter_sliced(int ncomp, int bytes, int64_t nt, int64_t nkept, int64_t npix, double padded) {
     const double hits = (double)nkept / (double)npix;
-    const bool shorter = bytes == 8 ? hits <= 300
-                                    : padded <= 24 || (padded < (ncomp == 1 ? 132 : 112) && nkept >= (1 << 19));
-    const bool few = npix <= 1024 && (ncomp == 1 ? hits >= (bytes == 8 ? 8192 : 4096) : hits >= 4096 && nkept >= (1 << 21));
     const double cached = (double)nt * bytes / (double)(1 << 27);   // of 128 MB
+    if (bytes == 4 && ncomp == 3)
+        return padded <= 24 || (hits < 128 && nkept >= (1 << 19)) || hits >= 4096 || cached > 1;
+    const bool shorter = bytes == 8 ? hits <= 300 : padded <= 24 || (padded < 132 && nkept >= (1 << 19));
+    const bool few = npix <= 1024 && (ncomp == 1 ? hits >= (bytes == 8 ? 8192 : 4096) : hits >= 4096 && nkept >= (1 << 21));
     return shorter || few || (cached > 1 && hits < 256 * cached);
 }
 

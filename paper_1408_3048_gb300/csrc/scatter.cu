@@ -257,17 +257,28 @@ __global__ void __launch_bounds__(WPB * 32, (sl_min_blocks<T, NC, WPB>())) slice
     }
 }
 
-// Warps per slice: enough of them for half the chip's warps, each with at least a batch of
-// steps.  (More parts shorten the last, partly filled wave of blocks but also the slices' runs:
-// four warps per slice on 8192 slices of 64 steps took 51 us, one 47.)  groups: of right-hand
-// sides, each a walk over every slice; a batch's warps have several loads in flight for a step
-// and fill the chip four times as early (512 slices of 64 steps, four groups of four columns:
-// one warp per slice, with two a batched solve took 2 % longer).
+// Warps per slice.  One column: enough of them for half the chip's warps, each with at least a
+// batch of steps.  (More parts shorten the last, partly filled wave of blocks but also the slices'
+// runs: four warps per slice on 8192 slices of 64 steps took 51 us, one 47.)
+// groups: of a batch's right-hand sides, each a walk over every slice by warps with several loads
+// in flight for a step.  Half as many of them are enough, and from a quarter on only long walks
+// gain, most of all by the first split, which changes the kernel (A x in us by parts, I/Q/U; 512
+// walks of 64 steps 1: 83, 4: 72, 8: 70; of 256 287, 203, 170; 1024 of 128 1: 259, 2: 227, 4: 187;
+// 2048 of 64 1: 158, 2: 160, of 128 323, 317, of 256 504, 498; T, of 64 128, 120, of 256 446, 369;
+// 4096 of 64 1: 253, 2: 282).
 int sliced_parts(const Plan& P, int groups) {
     const int64_t steps = P.sl_count > 0 ? P.sl_steps / P.sl_count : 0;
-    const int64_t enough = (int64_t)P.num_sms * (groups > 0 ? 8 : 32), walks = (int64_t)P.sl_count * std::max(groups, 1);
     int S = 1;
-    while (S < 32 && walks * S < enough && steps / (2 * S) >= SL_U) S *= 2;
+    if (groups == 0) {
+        while (S < 32 && (int64_t)P.sl_count * S < (int64_t)P.num_sms * 32 && steps / (2 * S) >= SL_U) S *= 2;
+        return S;
+    }
+    const int64_t walks = (int64_t)P.sl_count * groups;
+    while (S < 32 && walks * S < (int64_t)P.num_sms * 16) {
+        const int least = walks * S < (int64_t)P.num_sms * 8 ? SL_U : S == 1 && P.ncomp == 3 ? 64 : 32;
+        if (steps / (2 * S) < least) break;
+        S *= 2;
+    }
     return S;
 }
 

@@ -204,10 +204,10 @@ def test_interval_of_a_tiles_outputs_takes_one_tile(lib, lam, logs, length, tile
 
 
 def test_batched_scatter_of_few_pixels_fills_the_chip(lib):
-    """64 pixels of 8192 samples are 8 slices: with two columns 32 warps take parts of each, with 64
-    columns (16 groups of four) 16 of them."""
+    """64 pixels of 8192 samples are 8 slices: 32 warps take parts of each, for two columns and in
+    each of the 16 groups of 64."""
     p = Plan(lib, [1 << 18], 100, 1, side=8)
-    for R, grid, warps in ((2, 8, 32), (64, 4 * 16, 32)):
+    for R, grid, warps in ((2, 8, 32), (64, 8 * 16, 32)):
         name, blocks, _ = p.batch(R)[1][-1]
         assert "sliced_batch_parts_kernelIfLi1ELi4ELi%dE" % warps in name and blocks == grid, (R, name, blocks)
     p.close()
