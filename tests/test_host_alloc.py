@@ -162,11 +162,13 @@ def test_one_set_of_input_buffers_per_plan(lib):
 
 
 MANY_PSDS = r"""
-import resource, sys
+import sys
 sys.path[:0] = [{here!r}, {root!r}]
 import test_host_alloc as t
 L = t.load({so!r})
-rss = lambda: 1024 * resource.getrusage(resource.RUSAGE_SELF).ru_maxrss
+def rss():   # this process's peak (the resource module's figure includes its parent's)
+    with open("/proc/self/status") as f:
+        return 1024 * next(int(l.split()[1]) for l in f if l.startswith("VmHWM"))
 small = t.Plan(L, [20000], 1000, 1, npsd=2, fft_log2_f64=14, fft_log2_f32=14)
 small.close()
 base, dev = rss(), L.fake_live_bytes()
