@@ -737,7 +737,7 @@ __device__ __forceinline__ void split_chain(typename Cx<T>::type u1, typename Cx
 // f_knee = 1 to 2 Hz the FP64 product left 3e-15 to 1e-12 of the lowest modes as rounding, the
 // chain less than 2e-15.  So FP32 takes the chain throughout, FP64 and double-float for the
 // bins where H_k and H_{N-k} differ by more than a factor 1 / SPLIT_RATIO (f_knee = 2 Hz at 100
-// Hz: 1 bin in 20; A x of 2^22 I/Q/U samples 808 -> 809 us, the double-float residual
+// Hz: 1 bin in 20; A x of 2^22 I/Q/U samples 808 -> 811 us, the double-float residual
 // 476 -> 473).
 template <typename T>
 __device__ __forceinline__ void split_product(typename Cx<T>::type u1, typename Cx<T>::type u2, T a1, T a2, T b,
@@ -763,16 +763,19 @@ struct SplitRow {
         if constexpr (std::is_same<T, double>::value) return (int)v;
         else return (int)v.hi;
     }
+    // of a chained pair
+    __device__ __forceinline__ void chain(typename Cx<T>::type u1, typename Cx<T>::type u2, int k, T a1, T a2,
+                                          typename Cx<T>::type& V1, typename Cx<T>::type& V2) const {
+        const int m = k <= N / 2 ? k : N - k;
+        const T c = quarter[m];
+        split_chain<T>(u1, u2, k <= N / 2 ? c : -c, quarter[N / 2 - m], a1, k == 0 ? be[0] : a2, V1, V2);
+    }
     __device__ __forceinline__ void product(typename Cx<T>::type u1, typename Cx<T>::type u2, int k, T a1, T a2,
                                             typename Cx<T>::type& V1, typename Cx<T>::type& V2) const {
         const int m = k <= N / 2 ? k : N - k;
         const T b = be[m];   // requested with the others, ahead of the branch
-        if (m < kc) {
-            const T c = quarter[m];
-            split_chain<T>(u1, u2, k <= N / 2 ? c : -c, quarter[N / 2 - m], a1, k == 0 ? b : a2, V1, V2);
-        } else {
-            split_product<T>(u1, u2, a1, a2, b, V1, V2);
-        }
+        if (m < kc) chain(u1, u2, k, a1, a2, V1, V2);
+        else split_product<T>(u1, u2, a1, a2, b, V1, V2);
     }
 };
 
@@ -826,12 +829,27 @@ __device__ __forceinline__ void toeplitz_os_tile(const TzArgs<T>& A) {
         if (tid == 0) product(N / 2, __ldg(H + N / 2), __ldg(H + N / 2));
     } else {
         const SplitRow<T, N> row(A.H + tile.psd * split_size(N), A.twiddle, kc);
-        for (int k = tid; k <= N / 2; k += NT) {
+        auto put = [&](int k, C2 V1, C2 V2) {
             const int k2 = (N - k) & (N - 1);
-            C2 V1, V2;
-            row.product(a[pad<T>(k)], a[pad<T>(k2)], k, row.al[k], row.al[k2], V1, V2);
             a[pad<T>(k)] = V1;
             if (k2 != k) a[pad<T>(k2)] = V2;
+        };
+        // the chained bins in a loop of their own: with the branch inside one loop its code, unrolled,
+        // held up the double-float kernel (2^12 reals, 16 columns of 2^20 samples 497 us, this
+        // 466; folded throughout 465)
+        int k = tid;
+#pragma unroll 1
+        for (; k < kc; k += NT) {
+            const int k2 = (N - k) & (N - 1);
+            C2 V1, V2;
+            row.chain(a[pad<T>(k)], a[pad<T>(k2)], k, row.al[k], row.al[k2], V1, V2);
+            put(k, V1, V2);
+        }
+        for (; k <= N / 2; k += NT) {
+            const int k2 = (N - k) & (N - 1);
+            C2 V1, V2;
+            split_product<T>(a[pad<T>(k)], a[pad<T>(k2)], row.al[k], row.al[k2], row.be[k], V1, V2);
+            put(k, V1, V2);
         }
     }
     __syncthreads();
